@@ -307,16 +307,17 @@ typedef struct lfx_step_stats {
   float ms_assembly_kernels;    /* the assembly kernel's launches alone (CUDA events)          */
   int32_t n_assembly_launches;  /* launches of the assembly kernel in this step: element colours,
                                    chunk colours, or 1 for the persistent launch                */
-  float ms_spmv;                /* device time of a sample of the Arnoldi block SpMV launches of
-                                   the (inner) Krylov solve in this step: one in five, at most four
-                                   (CUDA events)                                                 */
+  float ms_spmv;                /* device time of Arnoldi block products of the (inner) Krylov solve
+                                   in this step: all of them where the persistent cycle runs (its own
+                                   clock), else a sample, one in five, at most four (CUDA events)  */
   int32_t n_spmv;               /* their number (FP64 matrix on the FP64 path, FP32 in mixed)   */
   int32_t newton_iterations;    /* Newton updates taken (fully implicit formulation), else 0    */
   float ms_newton_assembly;     /* device time of the Newton loop's assemblies: the residual
                                    checks and the Jacobians (CUDA events)                        */
-  int32_t n_fpass;              /* plain F passes of the preconditioner timed in this step (those
-                                   of its first application)                                     */
-  float ms_fpass_median;        /* their mean duration per pass (CUDA events)                     */
+  int32_t n_fpass;              /* plain F passes of the preconditioner timed in this step (all where
+                                   the persistent cycle runs, grid-wide wait included; else those of
+                                   its first application)                                        */
+  float ms_fpass_median;        /* their mean duration per pass                                   */
   int32_t assembly_mode;        /* LFX_ASM_* launch shape the step's assembly used                */
   int32_t reserved[2];
 } lfx_step_stats;

@@ -21,6 +21,7 @@
 #include "kernels.h"
 #include "lfx_internal.h"
 #include "amg.h"
+#include "cycle.h"
 #include "solver.h"
 
 namespace lfx {
@@ -955,6 +956,14 @@ lfx_status lfx_problem_create(const lfx_mesh *mesh, double rho, double mu, doubl
   LFX_CUDA_TRY(cudaMemcpy(pb->d_chunk_color_off.p, m.chunk_color_off.data(), sizeof(int32_t) * m.chunk_color_off.size(),
                           cudaMemcpyHostToDevice));
   pb->asm_mode = pb->asm_mode_newton = o.assembly;
+  // the row partition of the persistent Krylov cycle
+  if (o.s_smoother == LFX_SMOOTH_AMG && (m.n_comp == 1 || !o.batch_segmented)) {
+    int ctas = 0;
+    const CycleMap *map = nullptr;
+    if (o.precision == LFX_PREC_MIXED) LFX_TRY(cycle_ctas<float>(V, &ctas));
+    else LFX_TRY(cycle_ctas<double>(V, &ctas));
+    if (ctas > 0) LFX_TRY(mesh_cycle_map(m, ctas, &map));
+  }
   *out = pb.release();
   return LFX_OK;
 }
@@ -1458,6 +1467,7 @@ static lfx_status setup_asimple(lfx_state *s, ASimple<S, T> &pc) {
   lfx_problem *pb = s->pb;
   const lfx_options &o = pb->opt;
   const Mesh &m = pb->mesh->m;
+  if (m.n_comp == 1 || !o.batch_segmented) pc.plan_cycles(m);
   if (s->mixed())
     LFX_TRY(pc.setup_split(s->stream, s->view<float>(s->vals32), m.nnzb));   // from the high parts
   else
@@ -1506,6 +1516,13 @@ static lfx_status run_solve(lfx_state *s, double *x, bool x_zero, int *its, int 
     auto pc = [s, A](cudaStream_t q, const double *v, double *z, const KState *ks) {
       return s->pc64.apply(q, A, v, z, ks);
     };
+    if (s->pc64.cycle_ready() && !s->gm64.segmented()) {
+      s->gm64.whole_cycle = [s, A](cudaStream_t q, double *Vb, double *Zb, double *wk, double *xx, KState *ks, int m, int maxit) {
+        return s->pc64.cycle(q, A.rowptr, A.vals, Vb, Zb, wk, xx, ks, m, maxit);
+      };
+    } else {
+      s->gm64.whole_cycle = nullptr;
+    }
     return s->gm64.solve(st, A, pc, s->rhs.as<double>(), x, o.gmres_rtol, o.gmres_max_iters,
                          o.reorthogonalize != 0, kInnerLag, x_zero, its, rel);
   }
@@ -1526,6 +1543,15 @@ static lfx_status run_solve(lfx_state *s, double *x, bool x_zero, int *its, int 
     s->inner_cap = o.outer_max_iters + 2;
   }
   s->n_inner = 0;
+  s->gm32.whole_cycle = nullptr;
+  if (async_inner && o.smoother_bf16 && s->pcbf.cycle_ready())
+    s->gm32.whole_cycle = [s, A32](cudaStream_t q, float *Vb, float *Zb, float *wk, float *xx, KState *ks, int m, int maxit) {
+      return s->pcbf.cycle(q, A32.rowptr, A32.vals, Vb, Zb, wk, xx, ks, m, maxit);
+    };
+  else if (async_inner && !o.smoother_bf16 && s->pc32.cycle_ready())
+    s->gm32.whole_cycle = [s, A32](cudaStream_t q, float *Vb, float *Zb, float *wk, float *xx, KState *ks, int m, int maxit) {
+      return s->pc32.cycle(q, A32.rowptr, A32.vals, Vb, Zb, wk, xx, ks, m, maxit);
+    };
   auto inner = [s, A32, n, &o, adaptive, async_inner](cudaStream_t q, const double *v, double *z,
                                                       const KState *ks) -> lfx_status {
     LFX_TRY((launch_convert<double, float>(q, v, s->r32.as<float>(), n, ks)));
@@ -1875,7 +1901,9 @@ lfx_status lfx_step(lfx_state *s, lfx_step_stats *stats) {
   } else {
     s->newton_res.clear();
   }
-  if (s->mixed() && o.smoother_bf16) LFX_TRY(s->pcbf.queue_bulk_check(st));
+  if (!s->mixed()) LFX_TRY(s->pc64.queue_bulk_check(st));
+  else if (o.smoother_bf16) LFX_TRY(s->pcbf.queue_bulk_check(st));
+  else LFX_TRY(s->pc32.queue_bulk_check(st));
   LFX_CUDA_TRY(cudaEventRecord(s->e2, st));
   LFX_CUDA_TRY(cudaEventSynchronize(s->e2));
   s->assembled = false;
@@ -1886,9 +1914,9 @@ lfx_status lfx_step(lfx_state *s, lfx_step_stats *stats) {
     set_error("lfx_step: a grid-wide wait of the persistent assembly gave up; the state was not advanced");
     return LFX_ERR_TIMEOUT;
   }
-  if (s->pcbf.bulk_failed()) {
-    set_error("lfx_step: a wait for a staged tile of the velocity smoothing pass gave up; the state was not "
-              "advanced");
+  if (s->pcbf.bulk_failed() || s->pc32.bulk_failed() || s->pc64.bulk_failed()) {
+    set_error("lfx_step: a bounded wait of the linear solve (a staged tile of the velocity smoothing pass, or a "
+              "grid-wide wait of the persistent Krylov cycle) gave up; the state was not advanced");
     return LFX_ERR_TIMEOUT;
   }
   // history shift: the solution becomes level 0 (and d^{n+1} the displacement's level 0)
@@ -1922,12 +1950,15 @@ lfx_status lfx_step(lfx_state *s, lfx_step_stats *stats) {
       if (o.smoother_bf16) s->pcbf.read_f_timing(&stats->ms_fpass_median, &stats->n_fpass);
       else s->pc32.read_f_timing(&stats->ms_fpass_median, &stats->n_fpass);
       s->gm32.read_spmv_timing(&stats->ms_spmv, &stats->n_spmv);
+      s->pcbf.read_cycle_product(&stats->ms_spmv, &stats->n_spmv);
+      s->pc32.read_cycle_product(&stats->ms_spmv, &stats->n_spmv);
       int dummy = 0;
       float d2 = 0.0f;
       s->gmdd.read_spmv_timing(&d2, &dummy);
     } else {
       s->pc64.read_f_timing(&stats->ms_fpass_median, &stats->n_fpass);
       s->gm64.read_spmv_timing(&stats->ms_spmv, &stats->n_spmv);
+      s->pc64.read_cycle_product(&stats->ms_spmv, &stats->n_spmv);
     }
     stats->converged = rc == LFX_OK;
   }

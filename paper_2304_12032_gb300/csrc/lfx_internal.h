@@ -5,6 +5,8 @@
 #include <stdint.h>
 
 #include <string>
+#include <memory>
+#include <mutex>
 #include <vector>
 
 #include "lfx.h"
@@ -95,6 +97,14 @@ struct DBuf {
 };
 
 // ---------------------------------------------------------------- mesh (host + device)
+// The block rows dealt to `ctas` CTAs (CTA b: rows V b / ctas .. V (b + 1) / ctas), each with the list of
+// the rows of other CTAs that its blocks read (its halo, ascending), and every block's column as an index
+// into own rows followed by the halo.
+struct CycleMap {
+  int ctas = 0, max_rows = 0, max_loc = 0;   // max_loc: largest rows + halo (columns fit 16 bits up to 65536)
+  DBuf halo_off, halo, lcol;                 // int32 [ctas + 1], int32, uint16 [nnzb]
+};
+
 struct Mesh {
   int64_t V = 0, T = 0, F = 0, nnzb = 0;
   int n_flipped = 0;
@@ -155,12 +165,19 @@ struct Mesh {
   DBuf d_chunk_elem_off, d_chunk_pass_off, d_pass_code, d_pass_run_off, d_pass_ndiag, d_run_meta, d_run_block,
       d_run_node;
   DBuf d_ftile_row;
+  mutable std::mutex cycle_mu;
+  mutable std::vector<std::unique_ptr<CycleMap>> cycle_maps;   // built on first use, one per CTA count
   size_t device_bytes() const;
 };
 
 lfx_status build_mesh(const double *nodes, int64_t n_nodes, const int32_t *tets, int64_t n_tets,
                       const int32_t *bfaces, const int32_t *tags, int64_t n_bfaces, Mesh &m);
 lfx_status upload_mesh(Mesh &m);
+// the mesh's map for a CTA count (host lists, uploaded); it lives as long as the mesh
+lfx_status mesh_cycle_map(const Mesh &m, int ctas, const CycleMap **out);
+// its lists: halo rows of each CTA and local column indices
+void cycle_map_lists(const Mesh &m, int ctas, std::vector<int32_t> &halo_off, std::vector<int32_t> &halo,
+                     std::vector<uint16_t> &lcol, int *max_rows, int *max_loc);
 
 // ---------------------------------------------------------------- kernels' parameter blocks
 constexpr int kMaxRiis = 8;

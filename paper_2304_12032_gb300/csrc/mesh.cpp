@@ -4,6 +4,7 @@
 // transpose map, outward boundary faces, and a greedy element colouring so that elements of one
 // colour share no node and their block updates need no atomics.
 #include <algorithm>
+#include <thread>
 #include <cmath>
 #include <cstring>
 #include <numeric>
@@ -131,7 +132,12 @@ double signed_det(const double *x0, const double *x1, const double *x2, const do
 }  // namespace
 
 size_t Mesh::device_bytes() const {
-  return d_xyz.bytes + d_xyz_hi.bytes + d_xyz_lo.bytes + d_conn.bytes + d_slot.bytes + d_rowptr.bytes + d_col.bytes + d_diag.bytes +
+  size_t maps = 0;
+  {
+    std::lock_guard<std::mutex> lk(cycle_mu);
+    for (const auto &c : cycle_maps) maps += c->halo_off.bytes + c->halo.bytes + c->lcol.bytes;
+  }
+  return maps + d_xyz.bytes + d_xyz_hi.bytes + d_xyz_lo.bytes + d_conn.bytes + d_slot.bytes + d_rowptr.bytes + d_col.bytes + d_diag.bytes +
          d_trans.bytes + d_comp_off.bytes + d_node_old.bytes + d_first.bytes + d_color_elems.bytes +
          d_chunk_elem_off.bytes + d_chunk_pass_off.bytes + d_pass_code.bytes + d_pass_run_off.bytes +
          d_pass_ndiag.bytes + d_run_meta.bytes + d_run_block.bytes + d_run_node.bytes + d_ftile_row.bytes;
@@ -623,6 +629,74 @@ lfx_status upload_mesh(Mesh &m) {
   LFX_CUDA_TRY(cudaMemcpy(m.d_trans.p, m.trans_idx.data(), sizeof(int32_t) * m.nnzb, cudaMemcpyHostToDevice));
   LFX_CUDA_TRY(cudaMemcpy(m.d_comp_off.p, m.comp_off.data(), sizeof(int32_t) * m.comp_off.size(),
                           cudaMemcpyHostToDevice));
+  return LFX_OK;
+}
+
+void cycle_map_lists(const Mesh &m, int ctas, std::vector<int32_t> &halo_off, std::vector<int32_t> &halo,
+                     std::vector<uint16_t> &lcol, int *max_rows, int *max_loc) {
+  std::vector<std::vector<int32_t>> lists(ctas);
+  lcol.assign((size_t)std::max<int64_t>(m.nnzb, 1), 0);
+  const int nt = (int)std::min<unsigned>(std::max(1u, std::thread::hardware_concurrency()), 16u);
+  auto work = [&](int t) {
+    std::vector<int32_t> local((size_t)m.V, -1);
+    for (int b = t; b < ctas; b += nt) {
+      const int32_t r0 = (int32_t)(m.V * b / ctas), r1 = (int32_t)(m.V * (b + 1) / ctas);
+      std::vector<int32_t> &h = lists[b];
+      for (int32_t k = m.row_ptr[r0]; k < m.row_ptr[r1]; ++k) {
+        const int32_t c = m.col_idx[k];
+        if ((c < r0 || c >= r1) && local[c] < 0) {
+          local[c] = 0;
+          h.push_back(c);
+        }
+      }
+      std::sort(h.begin(), h.end());
+      for (size_t i = 0; i < h.size(); ++i) local[h[i]] = (int32_t)(r1 - r0 + (int64_t)i);
+      for (int32_t k = m.row_ptr[r0]; k < m.row_ptr[r1]; ++k) {
+        const int32_t c = m.col_idx[k];
+        lcol[k] = (uint16_t)(c >= r0 && c < r1 ? c - r0 : local[c]);   // (unused when max_loc exceeds 16 bits)
+      }
+      for (const int32_t c : h) local[c] = -1;
+    }
+  };
+  std::vector<std::thread> th;
+  for (int t = 1; t < nt; ++t) th.emplace_back(work, t);
+  work(0);
+  for (auto &t : th) t.join();
+  halo_off.assign(1, 0);
+  halo.clear();
+  *max_rows = *max_loc = 0;
+  for (int b = 0; b < ctas; ++b) {
+    const int rows = (int)(m.V * (b + 1) / ctas - m.V * b / ctas);
+    halo.insert(halo.end(), lists[b].begin(), lists[b].end());
+    halo_off.push_back((int32_t)halo.size());
+    *max_rows = std::max(*max_rows, rows);
+    *max_loc = std::max(*max_loc, rows + (int)lists[b].size());
+  }
+}
+
+lfx_status mesh_cycle_map(const Mesh &m, int ctas, const CycleMap **out) {
+  std::lock_guard<std::mutex> lk(m.cycle_mu);
+  for (const auto &c : m.cycle_maps)
+    if (c->ctas == ctas) {
+      *out = c.get();
+      return LFX_OK;
+    }
+  std::unique_ptr<CycleMap> c(new (std::nothrow) CycleMap);
+  if (!c) return LFX_ERR_OOM;
+  std::vector<int32_t> off, halo;
+  std::vector<uint16_t> lcol;
+  cycle_map_lists(m, ctas, off, halo, lcol, &c->max_rows, &c->max_loc);
+  auto up = [](DBuf &d, const void *src, size_t bytes) -> lfx_status {
+    LFX_TRY(d.alloc(std::max<size_t>(bytes, 16)));
+    if (bytes) LFX_CUDA_TRY(cudaMemcpy(d.p, src, bytes, cudaMemcpyHostToDevice));
+    return LFX_OK;
+  };
+  LFX_TRY(up(c->halo_off, off.data(), sizeof(int32_t) * off.size()));
+  LFX_TRY(up(c->halo, halo.data(), sizeof(int32_t) * halo.size()));
+  LFX_TRY(up(c->lcol, lcol.data(), sizeof(uint16_t) * lcol.size()));
+  c->ctas = ctas;
+  *out = c.get();
+  m.cycle_maps.push_back(std::move(c));
   return LFX_OK;
 }
 

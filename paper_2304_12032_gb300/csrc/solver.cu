@@ -19,10 +19,12 @@
 #include <type_traits>
 
 #include "amg.h"
+#include "cycle.h"
 #include "dd.h"
 #include "kernels.h"
 #include "pdl.h"
 #include "solver.h"
+#include "solver_dev.h"
 
 namespace lfx {
 
@@ -43,81 +45,6 @@ constexpr int kRowGroup = LFX_ROW_GROUP;   // lanes per block row in the row ker
 #ifndef LFX_U_GDC
 #define LFX_U_GDC 2
 #endif
-
-template <class T> struct Vec4T;
-template <> struct Vec4T<double> { using type = D4; };
-template <> struct Vec4T<float> { using type = F4; };
-
-// Arithmetic type of the vector kernels: FP32 vectors (the inner solve) are combined in FP32 and
-// only per-thread partial sums are widened to FP64 for the cross-thread reduction; FP64 vectors
-// stay FP64 throughout.  (FP64 instructions issue at 1/61 of the FP32 rate on this part, so an
-// FP64 accumulator would make the FP32 Krylov kernels arithmetic-bound.)
-template <class T, class X = T> struct AccT { using type = double; };
-template <> struct AccT<float, float> { using type = float; };
-
-template <class T>
-__device__ __forceinline__ typename Vec4T<T>::type ld4(const T *p, int64_t i) {
-  return reinterpret_cast<const typename Vec4T<T>::type *>(p)[i];
-}
-template <class T>
-__device__ __forceinline__ void st4(T *p, int64_t i, const typename Vec4T<T>::type &v) {
-  reinterpret_cast<typename Vec4T<T>::type *>(p)[i] = v;
-}
-
-// Two packed BF16 values to FP32 (exact: a BF16 value is the top half of its FP32 value).  Bit
-// operations on the integer pipe; the conversion instruction would take FP64-pipe issue slots.
-__device__ __forceinline__ void bf16x2_to_f32(uint32_t w, float &lo, float &hi) {
-  lo = __uint_as_float(w << 16);
-  hi = __uint_as_float(w & 0xffff0000u);
-}
-
-template <class S, class A>
-__device__ __forceinline__ void ld_block(const S *vals, int64_t k, A b[16]);
-template <>
-__device__ __forceinline__ void ld_block<double, double>(const double *vals, int64_t k, double b[16]) {
-  const double2 *p = reinterpret_cast<const double2 *>(vals + 16 * k);
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    double2 v = __ldg(p + i);
-    b[2 * i] = v.x;
-    b[2 * i + 1] = v.y;
-  }
-}
-template <>
-__device__ __forceinline__ void ld_block<float, float>(const float *vals, int64_t k, float b[16]) {
-  const float4 *p = reinterpret_cast<const float4 *>(vals + 16 * k);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float4 v = __ldg(p + i);
-    b[4 * i] = v.x;
-    b[4 * i + 1] = v.y;
-    b[4 * i + 2] = v.z;
-    b[4 * i + 3] = v.w;
-  }
-}
-template <>
-__device__ __forceinline__ void ld_block<__nv_bfloat16, float>(const __nv_bfloat16 *vals, int64_t k, float b[16]) {
-  const uint4 *p = reinterpret_cast<const uint4 *>(vals + 16 * k);
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    uint4 v = __ldg(p + i);
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) bf16x2_to_f32(w[q], b[8 * i + 2 * q], b[8 * i + 2 * q + 1]);
-  }
-}
-template <>
-__device__ __forceinline__ void ld_block<float, double>(const float *vals, int64_t k, double b[16]) {
-  const float4 *p = reinterpret_cast<const float4 *>(vals + 16 * k);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float4 v = __ldg(p + i);
-    b[4 * i] = v.x;
-    b[4 * i + 1] = v.y;
-    b[4 * i + 2] = v.z;
-    b[4 * i + 3] = v.w;
-  }
-}
 
 template <class A>
 __device__ __forceinline__ A group_sum(A v) {
@@ -193,20 +120,6 @@ __device__ __forceinline__ double cta_max(double v) {
   if (threadIdx.x == 0)
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s = fmax(s, red[i]);
   return s;
-}
-
-// a smoothing coefficient in the arithmetic type T (the FP32 kernels read the FP32 copy)
-template <class T>
-__device__ __forceinline__ T coef_t(const double &d, const float &) {
-  return (T)d;
-}
-template <>
-__device__ __forceinline__ float coef_t<float>(const double &, const float &f) {
-  return f;
-}
-
-__device__ __forceinline__ bool finished(const KState *st) {
-  return st != nullptr && *(volatile const int *)&st->done != 0;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -356,46 +269,6 @@ __global__ void reduce_kernel(const double *part, int n, double *out, int root) 
 //   velocity columns) with C appended (4).  Two storages: the full 4x4 blocks (BsrView) and the
 //   blocks stored apart (SplitView), where every pass over the matrix reads only the sub-block
 //   it needs.
-template <class S>
-struct SplitView {
-  int64_t V;
-  const int32_t *rowptr, *col, *diag, *trans;
-  const S *F;    // [nnzb][12]: F00 F01 F02 F10 F11 F12 F20 F21 F22 0 0 0
-  const S *G;    // [nnzb][4]:  G0 G1 G2 0
-  const S *DC;   // [nnzb][4]:  D0 D1 D2 C
-};
-
-// N consecutive values (N a multiple of 4) from an aligned record
-template <int N>
-__device__ __forceinline__ void ld_rec(const double *p, double *o) {
-#pragma unroll
-  for (int i = 0; i < N / 2; ++i) {
-    const double2 v = __ldg(reinterpret_cast<const double2 *>(p) + i);
-    o[2 * i] = v.x;
-    o[2 * i + 1] = v.y;
-  }
-}
-template <int N>
-__device__ __forceinline__ void ld_rec(const float *p, float *o) {
-#pragma unroll
-  for (int i = 0; i < N / 4; ++i) {
-    const float4 v = __ldg(reinterpret_cast<const float4 *>(p) + i);
-    o[4 * i] = v.x;
-    o[4 * i + 1] = v.y;
-    o[4 * i + 2] = v.z;
-    o[4 * i + 3] = v.w;
-  }
-}
-template <int N>
-__device__ __forceinline__ void ld_rec(const __nv_bfloat16 *p, float *o) {
-#pragma unroll
-  for (int i = 0; i < N / 4; ++i) {
-    const uint2 v = __ldg(reinterpret_cast<const uint2 *>(p) + i);
-    bf16x2_to_f32(v.x, o[4 * i], o[4 * i + 1]);
-    bf16x2_to_f32(v.y, o[4 * i + 2], o[4 * i + 3]);
-  }
-}
-
 template <class S, class T>
 __device__ __forceinline__ void ld_F(const BsrView<S> &A, int64_t k, T f[9]) {
   T b[16];
@@ -438,35 +311,48 @@ __device__ __forceinline__ void ld_DC(const SplitView<S> &A, int64_t k, T dc[4])
 }
 
 // Blocks stored apart (in the preconditioner's storage type S) from the FP64 or FP32 4x4 blocks.
-// Record slots 9..11 of an F sub-block: zero, except in BF16 storage, where slots 9 and 10 carry the
-// block's column index (low and high 16 bits) for the staged pass, which reads records only.
+// Record slots 9..11 of an F sub-block: in BF16 storage slots 9 and 10 carry the block's column index
+// (low and high 16 bits) for the staged pass, which reads records only; slot 11 (BF16 and FP32) the
+// column's local index in the persistent cycle's partition, which slot 3 of a G record carries too.
 template <class S>
-__device__ __forceinline__ void put_f_tail(S *rec, int32_t) {
+__device__ __forceinline__ void put_f_tail(S *rec, int32_t, uint16_t) {
   rec[9] = rec[10] = rec[11] = (S)0.0;
 }
 template <>
-__device__ __forceinline__ void put_f_tail<__nv_bfloat16>(__nv_bfloat16 *rec, int32_t c) {
+__device__ __forceinline__ void put_f_tail<float>(float *rec, int32_t, uint16_t l) {
+  rec[9] = rec[10] = 0.0f;
+  rec[11] = __uint_as_float((uint32_t)l);
+}
+template <>
+__device__ __forceinline__ void put_f_tail<__nv_bfloat16>(__nv_bfloat16 *rec, int32_t c, uint16_t l) {
   rec[9] = __ushort_as_bfloat16((unsigned short)((uint32_t)c & 0xffffu));
   rec[10] = __ushort_as_bfloat16((unsigned short)((uint32_t)c >> 16));
-  rec[11] = __ushort_as_bfloat16(0);
+  rec[11] = __ushort_as_bfloat16(l);
 }
+template <class S>
+__device__ __forceinline__ S g_tail(uint16_t) { return (S)0.0; }
+template <>
+__device__ __forceinline__ float g_tail<float>(uint16_t l) { return __uint_as_float((uint32_t)l); }
+template <>
+__device__ __forceinline__ __nv_bfloat16 g_tail<__nv_bfloat16>(uint16_t l) { return __ushort_as_bfloat16(l); }
 
 template <class S, class Src>
-__global__ void split_kernel(int64_t nnzb, const Src *__restrict__ vals, const int32_t *__restrict__ col, S *F, S *G,
-                             S *DC) {
+__global__ void split_kernel(int64_t nnzb, const Src *__restrict__ vals, const int32_t *__restrict__ col,
+                             const uint16_t *__restrict__ lcol, S *F, S *G, S *DC) {
   pdl_entry();
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nnzb; k += (int64_t)gridDim.x * blockDim.x) {
     Src b[16];
     ld_block<Src, Src>(vals, k, b);
+    const uint16_t l = lcol ? lcol[k] : (uint16_t)0;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
       for (int j = 0; j < 3; ++j) F[12 * k + 3 * i + j] = (S)b[4 * i + j];
-    put_f_tail<S>(F + 12 * k, col[k]);
+    put_f_tail<S>(F + 12 * k, col[k], l);
     G[4 * k] = (S)b[3];
     G[4 * k + 1] = (S)b[7];
     G[4 * k + 2] = (S)b[11];
-    G[4 * k + 3] = (S)0.0;
+    G[4 * k + 3] = g_tail<S>(l);
 #pragma unroll
     for (int i = 0; i < 4; ++i) DC[4 * k + i] = (S)b[12 + i];
   }
@@ -1111,48 +997,6 @@ __global__ void add_w_kernel(int64_t V, const T *d, T *x, const KState *st) {
   }
 }
 
-// ---- explicit CSR levels of the Schur AMG (scalar unknowns).  Values are stored in the
-// preconditioner's vector type T (FP32 for the mixed-precision inner solve, FP64 otherwise).
-template <class VT>
-struct CsrV {
-  int64_t n;
-  const int32_t *rp, *ci;
-  const VT *v;
-};
-
-// sum_k v[k] x[ci[k]*is + io] over the row, G lanes per row (lane = position in the group),
-// four nonzeros per lane in flight; the group's total is returned in every lane of the group.
-// Lanes with valid == false add nothing but take part in the shuffles.
-template <int G, class T>
-__device__ __forceinline__ typename AccT<T>::type csr_row_dot(const int32_t *__restrict__ rp,
-                                                              const int32_t *__restrict__ ci,
-                                                              const T *__restrict__ v, const T *x, int is, int io,
-                                                              int64_t row, int lane, bool valid) {
-  using A = typename AccT<T>::type;
-  A s = A(0);
-  if (valid) {
-    const int32_t k1 = __ldg(rp + row + 1);
-    int32_t k = __ldg(rp + row) + lane;
-    for (; k + 3 * G < k1; k += 4 * G) {
-      int32_t c[4];
-      T w[4], xv[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        c[u] = __ldg(ci + k + u * G);
-        w[u] = __ldg(v + k + u * G);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) xv[u] = x[(int64_t)c[u] * is + io];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) s += (A)w[u] * (A)xv[u];
-    }
-    for (; k < k1; k += G) s += (A)__ldg(v + k) * (A)x[(int64_t)__ldg(ci + k) * is + io];
-  }
-#pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
-}
-
 // out[i*os + oo] = (acc ? out : 0) + alpha * sum_j M_ij in[j*is + io]
 template <class T, int G>
 __global__ void __launch_bounds__(kThreads) csr_spmv_kernel(CsrV<T> M, const T *in, int is, int io, T *out, int os,
@@ -1220,32 +1064,6 @@ __global__ void __launch_bounds__(kThreads) csr_cheb_step_kernel(CsrV<T> M, cons
   }
 }
 
-// sum_k Minv[row][k] b[k*is+io] over one warp (eight columns per lane in flight)
-template <class T>
-__device__ __forceinline__ typename AccT<T>::type dense_row_dot(int64_t n, const T *__restrict__ Minv, const T *b,
-                                                                int is, int io, int64_t row, int lane, bool valid) {
-  using A = typename AccT<T>::type;
-  A s = A(0);
-  if (valid) {
-    const T *m = Minv + row * n;
-    int64_t k = lane;
-    for (; k + 7 * 32 < n; k += 8 * 32) {
-      T w[8], xv[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        w[u] = __ldg(m + k + u * 32);
-        xv[u] = b[(k + u * 32) * is + io];
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) s += (A)w[u] * (A)xv[u];
-    }
-    for (; k < n; k += 32) s += (A)__ldg(m + k) * (A)b[k * is + io];
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
-}
-
 // x[i*os+oo] = sum_k Minv[i][k] b[k*is+io]  (dense, n x n, row-major)
 template <class T>
 __global__ void __launch_bounds__(kThreads) dense_mv_kernel(int64_t n, const T *Minv, const T *b, int is, int io,
@@ -1262,30 +1080,6 @@ __global__ void __launch_bounds__(kThreads) dense_mv_kernel(int64_t n, const T *
 // ---- the coarse part of the Schur AMG V-cycle (levels 1..L-1) in ONE cooperative launch:
 // every phase is a grid-strided loop (a warp per matrix row), phases are separated by grid-wide
 // barriers.  Replaces ~20 tiny launches per V-cycle whose cost is mostly launch latency.
-template <class T>
-struct CoarseLevel {
-  int64_t n, nnext;
-  const int32_t *rp, *ci;
-  const T *v, *dinv;
-  const int32_t *Prp, *Pci;
-  const T *Pv;
-  const int32_t *Rrp, *Rci;
-  const T *Rv;
-  T *x, *b, *r, *d0, *d1, *rr;
-  T *xo;   // where the level's final iterate is left (d1 when one smoothing step is fused, else x)
-  typename AccT<T>::type init, c1[kMaxSmooth], c2[kMaxSmooth];   // (converted on the host)
-};
-constexpr int kMaxCoarse = 8;
-template <class T>
-struct CoarseArgs {
-  int L;            // levels in amg[] (level 0 is matrix-free and not part of this launch)
-  int s_steps;
-  typename AccT<T>::type alpha;
-  const T *coarse_inv;
-  int64_t nc;
-  CoarseLevel<T> lv[kMaxCoarse];
-};
-
 template <class T>
 __global__ void __launch_bounds__(kThreads) amg_coarse_kernel(const CoarseArgs<T> *__restrict__ args, const KState *st) {
   if (finished(st)) return;
@@ -2362,7 +2156,7 @@ lfx_status ASimple<S, T>::init_borrowed(int64_t V_, const SmootherConfig &cfg_, 
 template <class S, class T>
 size_t ASimple<S, T>::device_bytes() const {
   return dinvF.bytes + dinvS.bytes + X.bytes + D0.bytes + D1.bytes + R.bytes + W.bytes + coef.bytes + part.bytes +
-         sF.bytes + sG.bytes + sDC.bytes + berr.bytes;
+         sF.bytes + sG.bytes + sDC.bytes + berr.bytes + cyc_part.bytes + cyc_sync.bytes;
 }
 
 // Diagonals and (Chebyshev) eigenvalue estimates for the current matrix.
@@ -2439,7 +2233,8 @@ lfx_status ASimple<S, T>::setup_split_from(cudaStream_t st, const BsrView<Src> &
     nnz_split = nnzb;
   }
   const int g = (int)std::max<int64_t>(1, std::min<int64_t>((nnzb + kThreads - 1) / kThreads, 152 * 16));
-  pdl_launch(split_kernel<S, Src>, g, kThreads, 0, st, nnzb, A64.vals, A64.col, sF.as<S>(), sG.as<S>(), sDC.as<S>());
+  pdl_launch(split_kernel<S, Src>, g, kThreads, 0, st, nnzb, A64.vals, A64.col,
+             plan && plan->map ? plan->map->lcol.template as<uint16_t>() : nullptr, sF.as<S>(), sG.as<S>(), sDC.as<S>());
   note_launches(1);
   if (std::is_same<S, __nv_bfloat16>::value && !berr.p) {
     // error word of the staged velocity smoothing pass, and its host copy
@@ -2823,13 +2618,95 @@ lfx_status ASimple<S, T>::vcycle(cudaStream_t st, int l, const KState *ks) {
 }
 
 template <class S, class T>
+void ASimple<S, T>::plan_cycles(const Mesh &m) {
+  int dev = 0;
+  if (cfg.s_kind != LFX_SMOOTH_AMG || cfg.s_steps != 1 || cfg.f_steps < 2 || cudaGetDevice(&dev) != cudaSuccess) return;
+  if (!plan) plan = new CyclePlan;
+  if (plan->device == dev) return;
+  int ctas = 0;
+  const CycleMap *map = nullptr;
+  if (cycle_ctas<T>(V, &ctas) != LFX_OK || ctas < 1 || mesh_cycle_map(m, ctas, &map) != LFX_OK ||
+      plan_cycle<S, T>(V, m.nnzb, *map, plan) != LFX_OK) {
+    *plan = CyclePlan{};   // the step-by-step path runs
+    plan->device = dev;
+    clear_error();
+  }
+}
+
+template <class S, class T>
+bool ASimple<S, T>::cycle_ready() const {
+  const int L = (int)amg.size();
+  return plan && plan->rows_ctas > 0 && split && amg_ready && L >= 1 && L <= kMaxCoarse && (L == 1 || coarse_args.p);
+}
+
+template <class S, class T>
+lfx_status ASimple<S, T>::cycle(cudaStream_t st, const int32_t *rowptr, const T *A, T *Vb, T *Zb, T *wk, T *x, KState *ks,
+                                int m, int maxit) {
+  if (!cyc_sync.p) {
+    LFX_TRY(cyc_part.alloc(cycle_part_bytes(*plan)));
+    LFX_TRY(cyc_sync.alloc(sizeof(CycleSync)));
+    LFX_CUDA_TRY(cudaMemsetAsync(cyc_sync.p, 0, sizeof(CycleSync), st));
+    LFX_CUDA_TRY(cudaMallocHost(&cyc_host, sizeof(CycleSync)));
+    std::memset(cyc_host, 0, sizeof(CycleSync));
+  }
+  CycleArgs<S, T> a{};
+  a.V = V;
+  a.rowptr = rowptr;
+  a.F = sF.as<S>();
+  a.G = sG.as<S>();
+  a.DC = sDC.as<S>();
+  a.A = A;
+  a.dinvF = dinvF.as<T>();
+  a.dinvS = dinvS.as<T>();
+  a.cf = coef.as<SmoothCoef>();
+  a.f_steps = cfg.f_steps;
+  a.Q = R.as<T>();
+  a.D0 = D0.as<T>();
+  a.D1 = D1.as<T>();
+  a.X = X.as<T>();
+  a.W4 = W.as<T>();
+  a.rr = rr0.as<T>();
+  a.xp = Bs.as<T>();
+  a.pf = Bs.as<T>() + V;
+  a.t = Bs.as<T>() + 2 * V;
+  a.wk = wk;
+  a.L = (int)amg.size();
+  a.coarse_inv = coarse_inv.as<T>();
+  if (a.L >= 2) {
+    const AmgDevLevel &L0 = amg[0];
+    a.coarse = coarse_args.as<CoarseArgs<T>>();
+    a.R0 = CsrV<T>{L0.nnext, L0.Rrp.as<int32_t>(), L0.Rci.as<int32_t>(), L0.Rv.as<T>()};
+    a.P0 = CsrV<T>{V, L0.Prp.as<int32_t>(), L0.Pci.as<int32_t>(), L0.Pv.as<T>()};
+    a.b1 = amg[1].b.as<T>();
+    a.x1 = coarse_x();
+    a.alpha = (T)amg_alpha;
+  }
+  a.Vb = Vb;
+  a.Zb = Zb;
+  a.x = x;
+  a.ks = ks;
+  a.part = cyc_part.p;
+  a.part_n = cyc_part.as<double>() + cycle_part_norm_offset(*plan);
+  a.sync = cyc_sync.as<CycleSync>();
+  a.m = m;
+  a.maxit = maxit;
+  return launch_cycle<S, T>(st, *plan, a);
+}
+
+template <class S, class T>
 ASimple<S, T>::~ASimple() {
   for (cudaEvent_t e : fev) cudaEventDestroy(e);
+  delete plan;
+  if (cyc_host) cudaFreeHost(cyc_host);
   if (berr_host) cudaFreeHost(berr_host);
 }
 
 template <class S, class T>
 lfx_status ASimple<S, T>::queue_bulk_check(cudaStream_t st) {
+  if (cyc_sync.p) {
+    LFX_CUDA_TRY(cudaMemcpyAsync(cyc_host, cyc_sync.p, sizeof(CycleSync), cudaMemcpyDeviceToHost, st));
+    LFX_CUDA_TRY(cudaMemsetAsync(cyc_sync.p, 0, sizeof(CycleSync), st));
+  }
   if (!berr.p || !berr_host) return LFX_OK;
   LFX_CUDA_TRY(cudaMemcpyAsync(berr_host, berr.p, sizeof(int), cudaMemcpyDeviceToHost, st));
   LFX_CUDA_TRY(cudaMemsetAsync(berr.p, 0, sizeof(int), st));
@@ -2838,7 +2715,9 @@ lfx_status ASimple<S, T>::queue_bulk_check(cudaStream_t st) {
 
 template <class S, class T>
 bool ASimple<S, T>::bulk_failed() {
-  if (!berr_host || *berr_host == 0) return false;
+  const bool cycle_failed = cyc_host && cyc_host->error != 0;
+  if (cyc_host) cyc_host->error = 0;
+  if (!berr_host || *berr_host == 0) return cycle_failed;
   *berr_host = 0;
   return true;
 }
@@ -2857,9 +2736,21 @@ lfx_status ASimple<S, T>::read_f_timing(float *median_ms_per_pass, int *passes) 
   }
   n_fev = 0;
   std::sort(per.begin(), per.end());
+  if (cyc_host && cyc_host->n_f > 0) {   // the cycle's own clock: its passes, grid barrier included
+    if (median_ms_per_pass) *median_ms_per_pass = (float)((double)cyc_host->t_f * 1e-6 / cyc_host->n_f);
+    if (passes) *passes = cyc_host->n_f;
+    return LFX_OK;
+  }
   if (median_ms_per_pass) *median_ms_per_pass = per.empty() ? 0.0f : per[per.size() / 2];
   if (passes) *passes = (int)per.size() * std::max(cfg.f_steps - 2, 0);
   return LFX_OK;
+}
+
+template <class S, class T>
+void ASimple<S, T>::read_cycle_product(float *ms, int *count) const {
+  if (!cyc_host || cyc_host->n_spmv == 0) return;
+  *ms = (float)((double)cyc_host->t_spmv * 1e-6);
+  *count = cyc_host->n_spmv;
 }
 
 template <class S, class T>
@@ -2961,14 +2852,12 @@ lfx_status Gmres<S, T>::solve(cudaStream_t st, const BsrView<S> &A, const PrecFn
     pdl_launch(cycle_start_kernel, 1, kThreads, 0, st, pn, ng, ks);
     pdl_launch(scale_beta_kernel<T>, vg, kThreads, 0, st, w, Vb, n, ks);
     note_launches(2);
-    LFX_TRY(arnoldi_cycle(st, A, pc, restart, maxit, cgs2, lag));
-    pdl_launch(trisolve_kernel, 1, 32, 0, st, ks);
-    pdl_launch(update_x_kernel<T, T>, vg, kThreads, 0, st, Zb, n, x, n, ks);
+    LFX_TRY(run_cycle(st, A, pc, x, restart, maxit, cgs2, lag));
     // the true residual, which confirms convergence or starts the next cycle; one read of the
     // status header for both
     LFX_TRY(residual(st, A, x, b, w, pn, &ng));
     pdl_launch(reduce_kernel, 1, kThreads, 0, st, pn, ng, &ks->res, 1);
-    note_launches(3);
+    note_launches(1);
     LFX_CUDA_TRY(cudaMemcpyAsync(&hs, ks, offsetof(KState, H), cudaMemcpyDeviceToHost, st));
     LFX_CUDA_TRY(cudaStreamSynchronize(st));
     LFX_CUDA_TRY(cudaGetLastError());
@@ -3279,6 +3168,19 @@ lfx_status Gmres<S, T>::arnoldi_cycle(cudaStream_t st, const BsrView<S> &A, cons
   return LFX_OK;
 }
 
+// A cycle and the update of x: one launch where the owner provides it, else step by step.
+template <class S, class T>
+lfx_status Gmres<S, T>::run_cycle(cudaStream_t st, const BsrView<S> &A, const PrecFn<T> &pc, T *x, int m, int maxit,
+                                  bool cgs2, int lag) {
+  KState *ks = state.as<KState>();
+  if (whole_cycle && !cgs2 && r1.n_tags == 0) return whole_cycle(st, basis.as<T>(), zbasis.as<T>(), work.as<T>(), x, ks, m, maxit);
+  LFX_TRY(arnoldi_cycle(st, A, pc, m, maxit, cgs2, lag));
+  pdl_launch(trisolve_kernel, 1, 32, 0, st, ks);
+  pdl_launch(update_x_kernel<T, T>, vec_grid(n), kThreads, 0, st, zbasis.as<T>(), n, x, n, ks);
+  note_launches(2);
+  return LFX_OK;
+}
+
 template <class S, class T>
 lfx_status Gmres<S, T>::solve_inner(cudaStream_t st, const BsrView<S> &A, const PrecFn<T> &pc, const T *b, T *x,
                                     double rtol, const KState *outer, double lo, double hi, int maxit, bool cgs2,
@@ -3299,10 +3201,7 @@ lfx_status Gmres<S, T>::solve_inner(cudaStream_t st, const BsrView<S> &A, const 
   pdl_launch(inner_start_kernel, 1, kThreads, 0, st, pn, vg, ks, outer, rtol, lo, hi);
   pdl_launch(scale_beta_kernel<T>, vg, kThreads, 0, st, b, Vb, n, ks);
   note_launches(3);
-  LFX_TRY(arnoldi_cycle(st, A, pc, std::min(maxit, restart), maxit, cgs2, lag));
-  pdl_launch(trisolve_kernel, 1, 32, 0, st, ks);
-  pdl_launch(update_x_kernel<T, T>, vg, kThreads, 0, st, Zb, n, x, n, ks);
-  note_launches(2);
+  LFX_TRY(run_cycle(st, A, pc, x, std::min(maxit, restart), maxit, cgs2, lag));
   if (its_pinned) LFX_CUDA_TRY(cudaMemcpyAsync(its_pinned, &ks->total, sizeof(int), cudaMemcpyDeviceToHost, st));
   LFX_CUDA_TRY(cudaGetLastError());
   return LFX_OK;

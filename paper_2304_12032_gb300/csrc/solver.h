@@ -87,6 +87,9 @@ struct AmgDevLevel {
   double c1[kMaxSmooth] = {}, c2[kMaxSmooth] = {};
 };
 
+struct CyclePlan;
+struct CycleSync;
+
 template <class S, class T>
 struct ASimple {
   int64_t V = 0;
@@ -140,6 +143,17 @@ struct ASimple {
   // Work arrays carved from caller-provided device memory (no allocation); zeroed on st.
   static size_t scratch_bytes(int64_t V);
   lfx_status init_borrowed(int64_t V, const SmootherConfig &cfg, void *base, size_t cap, cudaStream_t st);
+  // One Krylov cycle as a single launch (cycle.cu): possible for sub-blocks stored apart with the Schur
+  // multigrid cycle of one smoothing step, when a CTA's share of the rows fits its shared memory.
+  // cycle(): m Arnoldi steps at most, for the operator A and v_0 in Vb, then x += sum_i y_i z_i.
+  CyclePlan *plan = nullptr;
+  DBuf cyc_part, cyc_sync;
+  CycleSync *cyc_host = nullptr;
+  void read_cycle_product(float *ms, int *count) const;   // its operator products since the last step
+  void plan_cycles(const Mesh &m);   // before setup_split, whose records carry the plan's local indices
+  bool cycle_ready() const;
+  lfx_status cycle(cudaStream_t st, const int32_t *rowptr, const T *A, T *Vb, T *Zb, T *wk, T *x, KState *ks, int m,
+                   int maxit);
   // Set-up on the full blocks A (the smoother then reads A's 4x4 blocks on every pass) ...
   lfx_status setup(cudaStream_t st, const BsrView<S> &A);
   // ... or on a copy of the FP64 blocks A64 converted to S with F, G and (D, C) stored apart, so
@@ -174,8 +188,13 @@ using PrecFn = std::function<lfx_status(cudaStream_t, const T *v, T *z, const KS
 template <class A, class B>
 lfx_status launch_convert(cudaStream_t st, const A *src, B *dst, int64_t n, const KState *ks);
 
+// One whole Arnoldi cycle from v_0 in Vb, the update of x included.
+template <class T>
+using CycleFn = std::function<lfx_status(cudaStream_t, T *Vb, T *Zb, T *work, T *x, KState *ks, int m, int maxit)>;
+
 template <class S, class T>
 struct Gmres {
+  CycleFn<T> whole_cycle;   // if set, runs a cycle of a single system (one Gram-Schmidt pass, no rank-one terms)
   int64_t V = 0, n = 0;
   int restart = 40;
   int nblk_dot = 0;
@@ -224,6 +243,8 @@ struct Gmres {
   void apply_rank1(cudaStream_t st, const T *x, T *y, double sign, const KState *ks);
   lfx_status residual(cudaStream_t st, const BsrView<S> &A, const T *x, const T *b, T *w, double *pn, int *ng);
   lfx_status timed_spmv(cudaStream_t st, const BsrView<S> &A, const T *z, T *w, const KState *ks);
+  lfx_status run_cycle(cudaStream_t st, const BsrView<S> &A, const PrecFn<T> &pc, T *x, int m, int maxit, bool cgs2,
+                       int lag);
   lfx_status arnoldi_cycle(cudaStream_t st, const BsrView<S> &A, const PrecFn<T> &pc, int m, int maxit, bool cgs2,
                            int lag);
   int n_seg = 0;

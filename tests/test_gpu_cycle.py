@@ -1,0 +1,53 @@
+"""The persistent Krylov cycle against the step-by-step launches of the same method (chosen by asking for a
+second Gram-Schmidt pass), at the sizes where its row partition changes shape: one CTA, 16, 8 or 4 lanes
+per row, a full grid with uneven shares, and hierarchies of one, two and more multigrid levels.
+
+Both solves stop at ||r|| <= 2e-12 ||b||, so they differ by at most 4e-12 times the amplification from
+residual to solution.  That amplification, taken from the benchmark flows' own tolerance sweeps, stays
+below 1e3 (velocity) and 1e4 (pressure of the pinned all-Dirichlet flow)."""
+import numpy as np
+import pytest
+
+from tests import cases as C
+
+pytestmark = pytest.mark.gpu
+
+
+def rel(a, b):
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("n,precision,opts", [
+    (2, "fp64", {}),                                    # 27 nodes: fewer rows than a CTA's least share
+    (6, "fp64", {}), (6, "mixed", {"smoother_bf16": 1}),   # the hierarchy is the dense inverse itself
+    (15, "fp64", {}), (16, "fp64", {}),                 # FP64: 16 lanes per row, then ten rows a warp
+    (12, "mixed", {"smoother_bf16": 1, "f_steps": 2}),  # two multigrid levels, the shortest smoother
+    (20, "mixed", {"smoother_bf16": 1}), (21, "mixed", {"smoother_bf16": 1}),   # FP32: 16 lanes, 8 lanes
+    (26, "mixed", {"smoother_bf16": 1}), (26, "mixed", {"smoother_bf16": 0}),   # 4 lanes
+    (26, "fp64", {"amg_coarse_size": 40}),              # three levels and more
+])
+def test_cycle_matches_step_by_step(n, precision, opts):
+    case = C.beltrami_case(n, seed=n)
+    out = []
+    for reorth in (0, 2 if precision == "mixed" else 1):
+        _, _, st = C.gpu_state(case, precision=precision, gmres_rtol=1e-12, reorthogonalize=reorth, **opts)
+        stats = st.step()
+        u, p = st.get()
+        out.append((u, p - p.mean(), stats))
+    (u, p, a), (ur, pr, b) = out
+    assert a["rel_residual"] <= 2e-12 and b["rel_residual"] <= 2e-12
+    assert rel(u, ur) < 4e-9 and rel(p, pr) < 4e-8
+    assert abs(a["iterations"] - b["iterations"]) <= 2 + b["iterations"] // 10
+    assert a["outer_iterations"] == b["outer_iterations"]
+
+
+def test_cycle_repeats_bit_for_bit():
+    """Fixed partitions and summation orders: the same step twice gives the same bits."""
+    case = C.beltrami_case(14, seed=3)
+    _, _, st = C.gpu_state(case, precision="mixed", smoother_bf16=1)
+    got = []
+    for _ in range(2):
+        st.set(case.u_hist, case.p_hist, case.t0)
+        st.step()
+        got.append(st.get())
+    assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
