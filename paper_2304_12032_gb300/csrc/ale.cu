@@ -9,7 +9,10 @@
 // graph), so the element -> block slot map of the assembly serves it unchanged.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "dd.h"
+#include "grid_wait.h"
 #include "kernels.h"
 #include "lfx_internal.h"
 #include "pdl.h"
@@ -83,6 +86,8 @@ __device__ __forceinline__ void cta_sum3(double a0, double a1, double a2, double
 struct CgState {
   double rz[3], rz0[3], alpha[3], beta[3];
   int iters, converged;
+  unsigned arrived;   // persistent solve: arrivals at its grid barrier
+  int error;          // a bounded wait gave up
 };
 
 // y = P K P x (P zeroes the fixed nodes), and partial sums of x . y per component
@@ -219,6 +224,194 @@ __global__ void cg_direction_kernel(int64_t V, const D4 *z, D4 *p, const CgState
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// The whole conjugate gradient iteration as one cooperative launch.  Step by step an iteration took
+// five launches, two of them single-thread sums of the partials (15 us each of 40 us at 15k nodes); here
+// every CTA owns a range of rows, their vectors (and their matrix entries, where they fit) stay in its
+// shared memory, only p goes through global memory, and an iteration costs three grid barriers.  Three
+// lanes share a row, one per displacement component: the FP64 pipe issues a warp instruction per about
+// 19 cycles of an SM whatever the number of active lanes, so the lanes are kept busy.
+// ------------------------------------------------------------------------------------------
+constexpr int kCgThreads = 512, kCgWarps = kCgThreads / 32, kCgRows = 10 * kCgWarps;
+constexpr int kCgSmem = 216 * 1024;
+constexpr int kCgMinRows = 8, kCgMaxCtas = 152;
+
+struct CgArgs {
+  int64_t V;
+  const int32_t *rowptr, *col;
+  const double *K, *dinv;
+  const uint8_t *fixed;
+  D4 *d, *p;
+  double *part;           // [2][3][CTAs]
+  CgState *cs;
+  double tol2;
+  int max_iters, max_rows;
+  uint32_t k_entries;     // matrix entries that fit beside the vectors
+};
+
+__host__ __device__ inline size_t cg_own_bytes(int rows) {
+  return ((size_t)rows * (12 * sizeof(double) + sizeof(double) + sizeof(int32_t)) + 64 + 15) & ~(size_t)15;
+}
+
+__global__ void __launch_bounds__(kCgThreads, 1) lifting_cg_kernel(const __grid_constant__ CgArgs A) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  __shared__ double red[kCgWarps][3], tot[3];
+  __shared__ int ok;
+  const unsigned ctas = gridDim.x, cta = blockIdx.x;
+  const int32_t r0 = (int32_t)(A.V * cta / ctas), n = (int32_t)(A.V * (cta + 1) / ctas) - r0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, c = lane % 3, first = warp * 10 + lane / 3;
+  const bool on = lane < 30;
+  double *x = reinterpret_cast<double *>(sm), *r = x + 3 * A.max_rows, *p = r + 3 * A.max_rows, *q = p + 3 * A.max_rows,
+         *dv = q + 3 * A.max_rows;
+  int32_t *rp = reinterpret_cast<int32_t *>(dv + A.max_rows);
+  double *sk = reinterpret_cast<double *>(sm + cg_own_bytes(A.max_rows));
+  int32_t *sc = reinterpret_cast<int32_t *>(sk + A.k_entries);
+  for (int i = tid; i <= n; i += kCgThreads) rp[i] = A.rowptr[r0 + i];
+  for (int i = tid; i < n; i += kCgThreads) {
+    dv[i] = A.fixed[r0 + i] ? 0.0 : A.dinv[r0 + i];
+    const D4 d = A.d[r0 + i];
+    x[3 * i] = d.x;
+    x[3 * i + 1] = d.y;
+    x[3 * i + 2] = d.z;
+  }
+  __syncthreads();
+  const int32_t k0 = rp[0];
+  const bool own_k = (uint32_t)(rp[n] - k0) <= A.k_entries;
+  if (own_k)
+    for (int32_t k = tid; k < rp[n] - k0; k += kCgThreads) {
+      sk[k] = A.K[k0 + k];
+      sc[k] = A.col[k0 + k];
+    }
+  const double *K = own_k ? sk - k0 : A.K;
+  const int32_t *col = own_k ? sc - k0 : A.col;
+  unsigned target = 0;
+  auto barrier = [&]() -> bool {
+    __syncthreads();
+    target += ctas;
+    if (tid == 0) {
+      arrive(&A.cs->arrived);
+      ok = wait_for(&A.cs->arrived, target, kWaitPolls);
+      if (!ok) atomicExch(&A.cs->error, 1);
+    }
+    __syncthreads();
+    return ok != 0;
+  };
+  // component c of sum_k K_k v(col k) for a row (fixed rows: 0; v vanishes at fixed nodes where it must)
+  auto product = [&](int row, const D4 *v) {
+    double a = 0.0;
+    if (dv[row] != 0.0) {
+      const int32_t e = rp[row + 1];
+      const double *w = reinterpret_cast<const double *>(v) + c;
+#pragma unroll 1
+      for (int32_t k = rp[row]; k < e; k += 5) {
+        double kv[5], xv[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u) {
+          const int32_t kk = min(k + u, e - 1);
+          kv[u] = K[kk];
+          xv[u] = w[4 * (int64_t)col[kk]];
+        }
+#pragma unroll
+        for (int u = 0; u < 5; ++u)
+          if (k + u < e) a += kv[u] * xv[u];
+      }
+    }
+    return a;
+  };
+  // this CTA's share of a sum per component, then (after a barrier) the sums over all CTAs
+  auto share = [&](double s, double *part) {
+    s += __shfl_down_sync(0xffffffffu, lane < 30 ? s : 0.0, 15);
+    const double a = __shfl_down_sync(0xffffffffu, s, 3), b = __shfl_down_sync(0xffffffffu, s, 6),
+                 d = __shfl_down_sync(0xffffffffu, s, 9), e = __shfl_down_sync(0xffffffffu, s, 12);
+    if (lane < 3) red[warp][lane] = s + a + b + d + e;
+    __syncthreads();
+    if (warp < 3) {
+      double t = lane < kCgWarps ? red[lane][warp] : 0.0;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) part[warp * ctas + cta] = t;
+    }
+  };
+  auto totals = [&](const double *part) {
+    if (warp < 3) {
+      double t = 0.0;
+      for (unsigned b = lane; b < ctas; b += 32) t += part[warp * ctas + b];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) tot[warp] = t;
+    }
+    __syncthreads();
+  };
+  double *gp = reinterpret_cast<double *>(A.p + r0);
+  double *part_a = A.part, *part_b = A.part + 3 * ctas;
+  __syncthreads();
+  // r = -(K d) on the free rows, z = D^-1 r, p = z
+  double s = 0.0;
+  for (int row = first; on && row < n; row += kCgRows) {
+    const double rv = -product(row, A.d), z = dv[row] * rv;
+    r[3 * row + c] = rv;
+    p[3 * row + c] = z;
+    gp[4 * row + c] = z;
+    s += rv * z;
+  }
+  share(s, part_b);
+  if (!barrier()) return;
+  totals(part_b);
+  double rz[3] = {tot[0], tot[1], tot[2]};
+  const double rz0[3] = {rz[0], rz[1], rz[2]};
+  int iters = 0, converged = (rz[0] <= 0.0 && rz[1] <= 0.0 && rz[2] <= 0.0) ? 1 : 0;
+  while (!converged) {
+    s = 0.0;
+    for (int row = first; on && row < n; row += kCgRows) {
+      const double a = product(row, A.p);
+      q[3 * row + c] = a;
+      s += p[3 * row + c] * a;
+    }
+    share(s, part_a);
+    if (!barrier()) return;
+    totals(part_a);
+    const double alpha = tot[c] > 0.0 ? rz[c] / tot[c] : 0.0;
+    s = 0.0;
+    for (int row = first; on && row < n; row += kCgRows) {
+      const int e = 3 * row + c;
+      const double rv = r[e] - alpha * q[e];
+      x[e] += alpha * p[e];
+      r[e] = rv;
+      s += rv * (dv[row] * rv);
+    }
+    share(s, part_b);
+    if (!barrier()) return;
+    totals(part_b);
+    bool done = true;
+    double beta = 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      if (i == c) beta = rz[i] > 0.0 ? tot[i] / rz[i] : 0.0;
+      rz[i] = tot[i];
+      if (rz[i] > A.tol2 * rz0[i]) done = false;
+    }
+    ++iters;
+    if (done || iters >= A.max_iters) {
+      converged = done ? 1 : 2;
+      break;
+    }
+    for (int row = first; on && row < n; row += kCgRows) {
+      const int e = 3 * row + c;
+      const double v = dv[row] * r[e] + beta * p[e];
+      p[e] = v;
+      gp[4 * row + c] = v;
+    }
+    if (!barrier()) return;
+  }
+  double *gd = reinterpret_cast<double *>(A.d + r0);
+  for (int row = first; on && row < n; row += kCgRows)
+    if (dv[row] != 0.0) gd[4 * row + c] = x[3 * row + c];
+  if (cta == 0 && tid == 0) {
+    A.cs->iters = iters;
+    A.cs->converged = converged;
+  }
+}
+
 // d at the listed nodes (fixed) = the given values; fixed flags set
 __global__ void set_fixed_kernel(int64_t n, const int32_t *node, const D4 *val, D4 *d, uint8_t *fixed) {
   pdl_entry();
@@ -308,6 +501,37 @@ lfx_status lifting_solve(cudaStream_t st, const LiftingView &L, int64_t n_fixed,
   CgState *cs = reinterpret_cast<CgState *>(L.cg_state);
   LFX_CUDA_TRY(cudaMemsetAsync(L.fixed, 0, (size_t)V, st));
   if (n_fixed > 0) pdl_launch(set_fixed_kernel, grid_of(n_fixed), kThr, 0, st, n_fixed, fixed_node, fixed_val, d, L.fixed);
+  int dev = 0, sms = 0, coop = 0;
+  LFX_CUDA_TRY(cudaGetDevice(&dev));
+  LFX_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  LFX_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+  const int ctas = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)sms, (int64_t)kCgMaxCtas, V / kCgMinRows}));
+  const int rows = (int)((V + ctas - 1) / ctas);
+  if (coop && cg_own_bytes(rows) <= (size_t)kCgSmem) {
+    CgArgs A{V, L.rowptr, L.col, L.K, L.dinv, L.fixed, d, L.p, L.part, cs, rtol * rtol, max_iters, rows, 0};
+    const size_t own = cg_own_bytes(rows), entry = sizeof(double) + sizeof(int32_t);
+    A.k_entries = (uint32_t)(((size_t)kCgSmem - own) / entry) & ~1u;
+    A.k_entries = std::min<uint32_t>(A.k_entries, (uint32_t)std::min<int64_t>(40LL * rows, 1 << 20));
+    LFX_CUDA_TRY(cudaMemsetAsync(cs, 0, sizeof(CgState), st));
+    LFX_CUDA_TRY(cudaFuncSetAttribute(lifting_cg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCgSmem));
+    void *kargs[] = {&A};
+    LFX_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)lifting_cg_kernel, dim3(ctas), dim3(kCgThreads), kargs,
+                                             own + entry * A.k_entries, st));
+    note_launches(1 + (n_fixed > 0));
+    CgState h{};
+    LFX_CUDA_TRY(cudaMemcpyAsync(&h, cs, sizeof(CgState), cudaMemcpyDeviceToHost, st));
+    LFX_CUDA_TRY(cudaStreamSynchronize(st));
+    if (iters_out) *iters_out = h.iters;
+    if (h.error) {
+      set_error("lifting: a grid-wide wait of the conjugate gradients gave up");
+      return LFX_ERR_TIMEOUT;
+    }
+    if (h.converged != 1) {
+      set_error("lifting: conjugate gradients did not converge in %d iterations", h.iters);
+      return LFX_ERR_NOT_CONVERGED;
+    }
+    return LFX_OK;
+  }
   pdl_launch(lap_residual_kernel, g, kThr, 0, st, V, L.rowptr, L.col, L.K, (const uint8_t *)L.fixed, (const D4 *)d, L.r);
   pdl_launch(cg_start_kernel, g, kThr, 0, st, V, L.dinv, (const uint8_t *)L.fixed, (const D4 *)L.r, L.z, L.p, L.part);
   pdl_launch(cg_scalar_kernel, 1, 32, 0, st, (const double *)L.part, g, cs, 0, rtol * rtol, max_iters);
@@ -340,7 +564,7 @@ lfx_status lifting_solve(cudaStream_t st, const LiftingView &L, int64_t n_fixed,
 }
 
 size_t lifting_cg_state_bytes() { return sizeof(CgState); }
-int lifting_part_entries(int64_t V) { return 3 * grid_of(V) + 8; }
+int lifting_part_entries(int64_t V) { return std::max(3 * grid_of(V), 6 * kCgMaxCtas) + 8; }
 
 lfx_status launch_move_nodes(cudaStream_t st, int64_t V, const D4 *ref, const D4 *d, D4 *x, float4 *hi, float4 *lo) {
   pdl_launch(move_nodes_kernel, grid_of(V), kThr, 0, st, V, ref, d, x, hi, lo);

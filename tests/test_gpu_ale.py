@@ -130,3 +130,28 @@ def test_translating_domain_is_the_fixed_domain_step_plus_v():
     assert np.abs(d - v * (t0 + dt)).max() <= 1e-12
     assert np.abs(um - v - uf).max() <= 1e-8 * np.abs(uf).max()
     assert np.abs(pm - pf).max() <= 1e-8 * np.abs(pf).max()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 9, 24, 60])
+def test_lifting_of_linear_boundary_data_is_linear(n):
+    """Linear displacements on the whole boundary extend to the linear field, whatever the partition of the
+    conjugate gradients: no free node (n = 1), one (2), fewer rows than CTAs (3), matrix entries in shared
+    memory (9, 24) and read from global memory (60).  The residual tolerance 1e-12, times at most about
+    (n / pi)^2 from residual to error, stays below 1e-9 of the field."""
+    from paper_2304_12032_gb300 import lfx as L
+    from synthetic import cube_kuhn
+
+    m = cube_kuhn(n, seed=n)
+    mesh = L.Mesh.from_synthetic(m)
+    prob = L.Problem(mesh, 1.0, 1.0, 1e-3, 1, [L.BC(tag=t, kind="nodal") for t in range(1, 7)], [],
+                     L.default_options(pin_pressure_node=0))
+    V = m.n_nodes
+    st = L.State(prob, np.zeros((1, V, 3)), np.zeros((1, V)), 0.0)
+    st.set_displacement(np.zeros((1, V, 3)))
+    d = m.nodes @ np.array([[0.02, 0.01, 0.0], [-0.01, 0.03, 0.0], [0.0, 0.02, -0.02]]) + 0.005
+    bd = np.unique(m.bfaces.ravel())
+    st.set_boundary_displacement(bd, d[bd])
+    st.step(allow_not_converged=True)
+    got, its = st.get_displacement()
+    assert np.abs(got - d).max() <= 1e-9 * np.abs(d).max()
+    assert (its == 0) == (n == 1)
