@@ -246,7 +246,8 @@ typedef struct lfx_options {
    * colour, each CTA scattering its elements' blocks), LFX_ASM_CHUNKS (compact 32-element chunks,
    * their blocks reduced in shared memory and written once per chunk, one launch per chunk colour),
    * LFX_ASM_PERSISTENT (the chunks in one cooperative launch, colours separated by bounded grid-wide
-   * waits; LFX_ERR_TIMEOUT from lfx_step if a wait gives up), or LFX_ASM_AUTO (default): the first
+   * waits, or, on meshes of up to about 190k tetrahedra, all chunks at once into a scratch and one wait
+   * before each block is summed over its chunks; LFX_ERR_TIMEOUT from lfx_step if a wait gives up), or LFX_ASM_AUTO (default): the first
    * assembly on the problem times each of the three on the device (two assemblies each) and the
    * problem keeps the fastest for all its states (lfx_problem_assembly_tuning reports it).  The
    * Newton system of the fully implicit formulation is timed and chosen apart from it, at its own

@@ -200,7 +200,7 @@ struct lfx_state {
   DBuf dhist[3], dnew, uale, xyz, xyz_hi, xyz_lo, geo64, geo_hi, geo_lo;
   DBuf lapK, lapDinv, lapFixed, lapR, lapZ, lapP, lapAp, lapPart, lapCg, bnd_node, bnd_val;
   // persistent assembly: grid-barrier counter and error word (device), the error word's host copy
-  DBuf asm_sync;
+  DBuf asm_sync, gather;   // (gather: the gathered assembly's scratch)
   int *asm_err_host = nullptr;
   int asm_mode_used = 0;
   bool force_timeout = false;   // tests: make the persistent assembly's first grid-wide wait run out
@@ -1182,9 +1182,14 @@ lfx_status lfx_state_device_bytes(const lfx_state *s, int64_t *bytes) {
              s->rhs_hi.bytes + s->rhs_lo.bytes + s->xe_hi.bytes + s->xe_lo.bytes + s->ub_hi.bytes + s->ub_lo.bytes +
              s->xs_hi.bytes + s->xs_lo.bytes;
   for (int l = 0; l < 3; ++l) b += s->hist[l].bytes;
-  b += s->io_u.bytes + s->io_p.bytes;
+  b += s->io_u.bytes + s->io_p.bytes + s->gather.bytes;
   *bytes = (int64_t)b;
   return LFX_OK;
+}
+
+// bytes of the gathered assembly's scratch (FP64 values, or double-float pairs: the same)
+static size_t gather_bytes(const Mesh &m) {
+  return m.blk_run.empty() ? 0 : sizeof(double) * (16 * m.blk_run.size() + 4 * (size_t)m.pass_diag_off.back());
 }
 
 // Assembly of the system for t^{n+1} = t + dt into vals64 / rhs, x0 = extrapolation.  With
@@ -1257,10 +1262,23 @@ static lfx_status assemble_system(lfx_state *s, bool apply_bcs, bool newton = fa
     A.uale = s->uale.as<D4>();
   }
   A.elist = m.d_color_elems.as<int32_t>();
-  const ChunkArgs CA{m.d_chunk_elem_off.as<int32_t>(), m.d_chunk_pass_off.as<int32_t>(), m.d_pass_code.as<uint16_t>(),
+  ChunkArgs CA{m.d_chunk_elem_off.as<int32_t>(), m.d_chunk_pass_off.as<int32_t>(), m.d_pass_code.as<uint16_t>(),
                      m.d_pass_run_off.as<int32_t>(), m.d_pass_ndiag.as<int32_t>(), m.d_run_meta.as<uint16_t>(),
                      m.d_run_block.as<int32_t>(), m.d_run_node.as<int32_t>()};
   const int n_cc = (int)m.chunk_color_off.size() - 1;
+  if (!m.blk_run.empty()) {
+    CA.diag_off = m.d_pass_diag_off.as<int32_t>();
+    CA.run_diag = m.d_run_diag.as<int32_t>();
+    CA.blk_off = m.d_blk_off.as<int32_t>();
+    CA.blk_run = m.d_blk_run.as<int32_t>();
+    CA.diag_idx = m.d_diag.as<int32_t>();
+    CA.n_chunks = (int64_t)m.chunk_elem_off.size() - 1;
+    CA.n_blocks = m.nnzb;
+    CA.n_runs = (int64_t)m.blk_run.size();
+    CA.n_diag = m.pass_diag_off.back();
+    if (!s->gather.p) LFX_TRY(s->gather.alloc(gather_bytes(m)));
+    CA.scratch = s->gather.p;
+  }
   if (mixed) A.bad = pb->n_bad > 0 ? pb->d_bad.as<uint8_t>() : nullptr;   // badly shaped: FP64 geometry
   if (!s->asm_sync.p) {
     LFX_TRY(s->asm_sync.alloc(64));
@@ -1411,6 +1429,8 @@ int64_t lfx_internal_state_bytes_estimate(const lfx_problem *pb, int64_t *V_out,
   if (sigma_out) *sigma_out = sigma;
   const int64_t v64 = 32 * V, v32 = 16 * V;
   int64_t b = (sigma + 3) * v64 + 64 * (int64_t)pb->dir_node.size() + 8 * m.n_comp;
+  b += (int64_t)gather_bytes(m);                             // gathered assembly
+  b += 9 * 152 * 8 * 65;                                     // partial sums of the persistent Krylov cycle
   b += sigma * v64;                                          // caller-layout staging (history in, solution out)
   b += 128 * nnzb;                                           // FP64 or double-float matrix
   const int64_t amg = o.s_smoother == LFX_SMOOTH_AMG ? 300 * V + 8LL * o.amg_coarse_size * o.amg_coarse_size : 0;

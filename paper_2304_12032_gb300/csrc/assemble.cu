@@ -942,13 +942,50 @@ __device__ void geom_load_range(const AssembleArgs &A, int64_t T, int64_t e0, in
   }
 }
 
+// Gathered form: where a run's (or a diagonal run's right-hand-side) values go in the scratch, and the
+// sum of them afterwards.
+template <class R> struct Gather;
+template <>
+struct Gather<double> {
+  static __device__ __forceinline__ double *at(const ChunkArgs &C, int64_t i, bool is_rhs) {
+    return static_cast<double *>(C.scratch) + (is_rhs ? 16 * C.n_runs : 0) + i;
+  }
+  static __device__ __forceinline__ void store(const ChunkArgs &C, int64_t i, bool is_rhs, const double v[4]) {
+    double2 *p = reinterpret_cast<double2 *>(at(C, i, is_rhs));
+    p[0] = make_double2(v[0], v[1]);
+    p[1] = make_double2(v[2], v[3]);
+  }
+  static __device__ __forceinline__ void load(const ChunkArgs &C, int64_t i, bool is_rhs, double v[4]) {
+    const double2 *p = reinterpret_cast<const double2 *>(at(C, i, is_rhs));
+    const double2 a = __ldcg(p), b = __ldcg(p + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+  }
+};
+template <>
+struct Gather<dd> {
+  static __device__ __forceinline__ float *at(const ChunkArgs &C, int64_t i, bool is_rhs) {
+    return static_cast<float *>(C.scratch) + (is_rhs ? 16 * C.n_runs : 0) + i;
+  }
+  static __device__ __forceinline__ int64_t low(const ChunkArgs &C) { return 16 * C.n_runs + 4 * C.n_diag; }
+  static __device__ __forceinline__ void store(const ChunkArgs &C, int64_t i, bool is_rhs, const dd v[4]) {
+    float *p = at(C, i, is_rhs);
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0].hi, v[1].hi, v[2].hi, v[3].hi);
+    *reinterpret_cast<float4 *>(p + low(C)) = make_float4(v[0].lo, v[1].lo, v[2].lo, v[3].lo);
+  }
+  static __device__ __forceinline__ void load(const ChunkArgs &C, int64_t i, bool is_rhs, dd v[4]) {
+    const float *p = at(C, i, is_rhs);
+    const float4 h = __ldcg(reinterpret_cast<const float4 *>(p)), l = __ldcg(reinterpret_cast<const float4 *>(p + low(C)));
+    v[0] = dd(h.x, l.x); v[1] = dd(h.y, l.y); v[2] = dd(h.z, l.z); v[3] = dd(h.w, l.w);
+  }
+};
+
 // The chunks c0 + blockIdx.x, c0 + blockIdx.x + gridDim.x, ... (< c1).  Each chunk's slot codes,
 // run tables and pass offsets are staged in shared memory at its start with loads that do not
 // wait on one another (its geometry loads among them), and the next chunk's offsets are loaded
 // while this one is processed, so that no phase waits on a chain of dependent global loads; its
 // node fields and geometry are prefetched into L2 during this chunk's first pass, its tables
 // during the second.
-template <class R, class S, bool IMPL>
+template <class R, class S, bool IMPL, bool kGather = false>
 __device__ __forceinline__ void chunk_range(const AssembleArgs &A, const PhysParams &P, const PhysR<R> &Q,
                                             const ChunkArgs &C, int64_t c0, int64_t c1, S *vals,
                                             ChunkShared<R, IMPL> &cs) {
@@ -993,7 +1030,7 @@ __device__ __forceinline__ void chunk_range(const AssembleArgs &A, const PhysPar
     else if (t < kElems && e0 + t < e1) geom_phase<R>(A, e0 + t, t, sh);
     __syncthreads();
     // the blocks (and rows) this chunk adds to, into L2 ahead of its reduction phases
-    for (int r = t; r < nrun; r += kCta) {
+    for (int r = t; !kGather && r < nrun; r += kCta) {
       const uint32_t meta = cs.meta[r];
       if ((meta >> 14) & 1) continue;
       const int64_t k = (int64_t)cs.block[r] * 16;
@@ -1105,7 +1142,12 @@ __device__ __forceinline__ void chunk_range(const AssembleArgs &A, const PhysPar
           const uint32_t meta = cs.meta[run];
           first[i] = (meta >> 14) & 1;
           is_rhs[i] = !blk_item;
-          where[i] = blk_item ? (int64_t)cs.block[run] * 16 + v0 : 4 * (int64_t)cs.node[run];
+          if constexpr (kGather) {
+            where[i] = blk_item ? (int64_t)(rb + run) * 16 + v0 : 4 * (int64_t)(C.diag_off[p0 + pi] + run - r0);
+            first[i] = true;
+          } else {
+            where[i] = blk_item ? (int64_t)cs.block[run] * 16 + v0 : 4 * (int64_t)cs.node[run];
+          }
           if (!first[i]) old[i] = Out::load(A, vals, where[i], is_rhs[i]);
           const int st0 = meta & 0xff, len = (meta >> 8) & 63;
 #pragma unroll
@@ -1117,7 +1159,10 @@ __device__ __forceinline__ void chunk_range(const AssembleArgs &A, const PhysPar
         }
 #pragma unroll
         for (int i = 0; i < kItemsInFlight; ++i)
-          if (where[i] >= 0) Out::store(A, vals, where[i], is_rhs[i], sum[i], old[i], first[i]);
+          if (where[i] >= 0) {
+            if constexpr (kGather) Gather<R>::store(C, where[i], is_rhs[i], sum[i]);
+            else Out::store(A, vals, where[i], is_rhs[i], sum[i], old[i], first[i]);
+          }
       }
       __syncthreads();   // (the last one also frees the staged tables for the next chunk)
     }
@@ -1138,6 +1183,16 @@ __device__ __forceinline__ void chunk_range(const AssembleArgs &A, const PhysPar
             for (int bb = 0; bb < 4; ++bb)
 #pragma unroll
               for (int i = 0; i < 4; ++i) sum[i] = (k == 0 && bb == 0) ? cs.n.ext[l2][a][0][i] : acc(sum[i], cs.n.ext[l2][a][bb][i]);
+          }
+          if constexpr (kGather) {
+            // (written before the CTA's last barrier by one of its threads)
+            const int64_t at = 4 * (int64_t)(C.diag_off[p0 + pi] + j);
+            R row[4];
+            Gather<R>::load(C, at, true, row);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) row[i] = acc(row[i], sum[i]);
+            Gather<R>::store(C, at, true, row);
+            continue;
           }
           const int64_t where = 4 * (int64_t)cs.node[r0 + j];
           const typename Out::Old old = Out::load(A, vals, where, true);
@@ -1209,6 +1264,40 @@ __global__ void __launch_bounds__(kCta, IMPL ? 1 : MinCtas<R>::value) assemble_c
     if (c + 1 < n_colors &&
         !grid_barrier(barrier, (unsigned)(c + 1) * gridDim.x + unreachable, err, max_spins))
       return;
+  }
+}
+
+// The gathered form of the persistent launch, for meshes whose chunk colours hold fewer chunks than the
+// GPU runs at once (a 19k-tetrahedron mesh: 590 chunks in 20 colours, of which 456 fit).  Coloured, a
+// chunk's 20 us of latency is paid once per colour; here all chunks run at once into the scratch, one
+// grid-wide wait, and every block is the sum of its runs in chunk order: the colours' order, so the
+// result is the same bit for bit (the Newton right-hand side apart, whose shares join per chunk).  ms per
+// step, coloured and gathered: 3k tetrahedra FP64 1.54 and 1.12, 19k mixed 3.28 and 3.00, 60k FP64 5.66 and
+// 5.13, 100k FP64 8.29 and 7.98, 150k mixed with Newton 16.1 and 13.6.
+template <class R, class S, bool IMPL>
+__global__ void __launch_bounds__(kCta, IMPL ? 1 : MinCtas<R>::value) assemble_chunks_gather_kernel(
+    AssembleArgs A, PhysParams P, PhysR<R> Q, ChunkArgs C, S *vals, unsigned *barrier, int *err, unsigned unreachable,
+    unsigned max_spins) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  chunk_range<R, S, IMPL, true>(A, P, Q, C, 0, C.n_chunks, vals, *reinterpret_cast<ChunkShared<R, IMPL> *>(smem_raw));
+  if (!grid_barrier(barrier, gridDim.x + unreachable, err, max_spins)) return;
+  using Out = AccumOut<S, R>;
+  // a quarter of a block (or a row's right-hand side, from its diagonal block's runs) per item
+  const int64_t n = 4 * C.n_blocks + A.n_nodes;
+  for (int64_t j = blockIdx.x * (int64_t)kCta + threadIdx.x; j < n; j += (int64_t)gridDim.x * kCta) {
+    const bool is_rhs = j >= 4 * C.n_blocks;
+    const int64_t k = is_rhs ? C.diag_idx[j - 4 * C.n_blocks] : j >> 2;
+    const int32_t q0 = C.blk_off[k], q1 = C.blk_off[k + 1];
+    R sum[4] = {cst<R>(0.0), cst<R>(0.0), cst<R>(0.0), cst<R>(0.0)};
+    for (int32_t q = q0; q < q1; ++q) {
+      const int32_t run = C.blk_run[q];
+      R v[4];
+      Gather<R>::load(C, is_rhs ? 4 * (int64_t)C.run_diag[run] : 16 * (int64_t)run + 4 * (j & 3), is_rhs, v);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) sum[i] = q == q0 ? v[i] : acc(sum[i], v[i]);
+    }
+    const int64_t where = is_rhs ? 4 * (j - 4 * C.n_blocks) : 16 * k + 4 * (j & 3);
+    Out::store(A, vals, where, is_rhs, sum, typename Out::Old(), true);
   }
 }
 
@@ -1555,10 +1644,40 @@ lfx_status launch_persistent_impl(cudaStream_t st, const AssembleArgs &A, const 
   return LFX_OK;
 }
 
+template <class R, class S, bool IMPL>
+lfx_status launch_gather_impl(cudaStream_t st, const AssembleArgs &A, const PhysParams &P, const ChunkArgs &C, S *vals,
+                              unsigned *barrier, int *err, bool force_timeout) {
+  const PhysR<R> Q = phys_r<R>(P);
+  const size_t smem = sizeof(ChunkShared<R, IMPL>);
+  int dev = 0, nsm = 152, per_sm = 0, coop = 0;
+  LFX_CUDA_TRY(cudaGetDevice(&dev));
+  LFX_CUDA_TRY(cudaFuncSetAttribute(assemble_chunks_gather_kernel<R, S, IMPL>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  LFX_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  LFX_CUDA_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+  LFX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, assemble_chunks_gather_kernel<R, S, IMPL>, kCta, smem));
+  if (!coop || per_sm < 1) {
+    set_error("persistent assembly: cooperative launch unavailable");
+    return LFX_ERR_CUDA;
+  }
+  LFX_CUDA_TRY(cudaMemsetAsync(barrier, 0, sizeof(unsigned), st));
+  LFX_CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
+  unsigned unreachable = force_timeout ? 1u : 0u, max_spins = force_timeout ? (1u << 12) : kBarrierSpins;
+  void *args[] = {(void *)&A,    (void *)&P,       (void *)&Q,   (void *)&C,           (void *)&vals,
+                  (void *)&barrier, (void *)&err, (void *)&unreachable, (void *)&max_spins};
+  LFX_CUDA_TRY(cudaLaunchCooperativeKernel((void *)assemble_chunks_gather_kernel<R, S, IMPL>, dim3(nsm * per_sm), dim3(kCta),
+                                           args, smem, st));
+  note_launches(1);
+  return LFX_OK;
+}
+
 template <class R, class S>
 lfx_status launch_assemble_persistent(cudaStream_t st, const AssembleArgs &A, const PhysParams &P, const ChunkArgs &C,
                                       const int32_t *d_chunk_color_off, int n_colors, S *vals, unsigned *barrier,
                                       int *err, bool force_timeout, bool newton) {
+  if (C.scratch)
+    return newton ? launch_gather_impl<R, S, true>(st, A, P, C, vals, barrier, err, force_timeout)
+                  : launch_gather_impl<R, S, false>(st, A, P, C, vals, barrier, err, force_timeout);
   return newton ? launch_persistent_impl<R, S, true>(st, A, P, C, d_chunk_color_off, n_colors, vals, barrier, err,
                                                      force_timeout)
                 : launch_persistent_impl<R, S, false>(st, A, P, C, d_chunk_color_off, n_colors, vals, barrier, err,

@@ -54,6 +54,13 @@ struct ChunkArgs {
   const int32_t *run_off, *ndiag;
   const uint16_t *meta;
   const int32_t *block, *node;
+  // Gathered form of the persistent launch (scratch null: the coloured form): every run's 16 block
+  // values and every diagonal run's 4 right-hand-side values in scratch, diagonal runs numbered from
+  // diag_off[pass]; then each block (and row) is the sum of its runs blk_run[blk_off[k] ..] in order.
+  const int32_t *diag_off, *run_diag, *blk_off, *blk_run, *diag_idx;   // run_diag: number of a diagonal run
+  int64_t n_chunks, n_blocks, n_runs;
+  void *scratch;             // R values: [n_runs][16], [n_diag][4]; double-float: high parts, then low parts
+  int64_t n_diag;
 };
 constexpr int kGeoValues = 24;
 

@@ -140,6 +140,11 @@ struct Mesh {
   std::vector<uint16_t> run_meta;        // slot start (bits 0-7) | length (8-13) | first writer (14) | diagonal (15)
   std::vector<int32_t> run_block;        // [runs] block index in the pattern
   std::vector<int32_t> run_node;         // [runs] node of a diagonal run (its rhs row), else -1
+  // gathered assembly (meshes of at most kGatherChunks chunks): first diagonal run of each pass, and
+  // the runs of every block, ascending
+  std::vector<int32_t> pass_diag_off;    // [n_passes+1]
+  std::vector<int32_t> run_diag;         // [runs] number of a diagonal run
+  std::vector<int32_t> blk_off, blk_run; // [nnzb+1], [runs]
   // tiles of the staged velocity smoothing pass: consecutive block rows, at most kFTileRows rows and
   // kFTileBlocks blocks each ([n_tiles+1] row offsets; empty when some row alone exceeds the limit)
   std::vector<int32_t> ftile_row;
@@ -165,6 +170,7 @@ struct Mesh {
   DBuf d_chunk_elem_off, d_chunk_pass_off, d_pass_code, d_pass_run_off, d_pass_ndiag, d_run_meta, d_run_block,
       d_run_node;
   DBuf d_ftile_row;
+  DBuf d_pass_diag_off, d_run_diag, d_blk_off, d_blk_run;
   mutable std::mutex cycle_mu;
   mutable std::vector<std::unique_ptr<CycleMap>> cycle_maps;   // built on first use, one per CTA count
   size_t device_bytes() const;
@@ -197,6 +203,10 @@ struct PhysParams {
 };
 
 constexpr int kChunkElems = 32;     // elements per chunk (one CTA pass of the assembly kernels)
+// Meshes of up to this many chunks are assembled by gathering (when the persistent launch is chosen):
+// below it the chunk colours hold fewer chunks than the GPU runs at once, so that colour by colour most
+// of it idles.  The scratch is about 26 KB per chunk (FP64 or double-float), 160 MB at the limit.
+constexpr int kGatherChunks = 6144;
 constexpr int kChunkMaxPasses = 8;  // passes of 4 kChunkElems slots a chunk may take (the kernels stage
                                     // a chunk's slot codes for this many in shared memory)
 // tile limits of the staged velocity smoothing pass (its CTA handles kFTileRows rows with 4 lanes

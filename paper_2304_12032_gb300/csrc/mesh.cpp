@@ -140,7 +140,8 @@ size_t Mesh::device_bytes() const {
   return maps + d_xyz.bytes + d_xyz_hi.bytes + d_xyz_lo.bytes + d_conn.bytes + d_slot.bytes + d_rowptr.bytes + d_col.bytes + d_diag.bytes +
          d_trans.bytes + d_comp_off.bytes + d_node_old.bytes + d_first.bytes + d_color_elems.bytes +
          d_chunk_elem_off.bytes + d_chunk_pass_off.bytes + d_pass_code.bytes + d_pass_run_off.bytes +
-         d_pass_ndiag.bytes + d_run_meta.bytes + d_run_block.bytes + d_run_node.bytes + d_ftile_row.bytes;
+         d_pass_ndiag.bytes + d_run_meta.bytes + d_run_block.bytes + d_run_node.bytes + d_ftile_row.bytes + d_pass_diag_off.bytes +
+         d_run_diag.bytes + d_blk_off.bytes + d_blk_run.bytes;
 }
 
 lfx_status build_mesh(const double *nodes, int64_t n_nodes, const int32_t *tets_in, int64_t n_tets,
@@ -544,6 +545,20 @@ lfx_status build_mesh(const double *nodes, int64_t n_nodes, const int32_t *tets_
     }
   }
 
+  if ((int64_t)m.chunk_elem_off.size() - 1 <= kGatherChunks) {
+    m.pass_diag_off.assign(1, 0);
+    for (const int32_t d : m.pass_ndiag) m.pass_diag_off.push_back(m.pass_diag_off.back() + d);
+    m.run_diag.assign(m.run_block.size(), -1);
+    for (size_t p = 0; p < m.pass_ndiag.size(); ++p)
+      for (int32_t d = 0; d < m.pass_ndiag[p]; ++d) m.run_diag[m.pass_run_off[p] + d] = m.pass_diag_off[p] + d;
+    m.blk_off.assign((size_t)m.nnzb + 1, 0);
+    for (const int32_t b : m.run_block) ++m.blk_off[b + 1];
+    for (int64_t k = 0; k < m.nnzb; ++k) m.blk_off[k + 1] += m.blk_off[k];
+    std::vector<int32_t> at(m.blk_off.begin(), m.blk_off.end() - 1);
+    m.blk_run.resize(m.run_block.size());
+    for (size_t r = 0; r < m.run_block.size(); ++r) m.blk_run[at[m.run_block[r]]++] = (int32_t)r;
+  }
+
   // ---- boundary faces: internal numbering, outward orientation from the owning tetrahedron
   m.bfaces.resize(3 * F);
   m.btags.assign(tags_in, tags_in + F);
@@ -608,6 +623,10 @@ lfx_status upload_mesh(Mesh &m) {
   LFX_TRY(up(m.d_run_meta, m.run_meta.data(), sizeof(uint16_t) * m.run_meta.size()));
   LFX_TRY(up(m.d_run_block, m.run_block.data(), sizeof(int32_t) * m.run_block.size()));
   LFX_TRY(up(m.d_run_node, m.run_node.data(), sizeof(int32_t) * m.run_node.size()));
+  LFX_TRY(up(m.d_pass_diag_off, m.pass_diag_off.data(), sizeof(int32_t) * m.pass_diag_off.size()));
+  LFX_TRY(up(m.d_run_diag, m.run_diag.data(), sizeof(int32_t) * m.run_diag.size()));
+  LFX_TRY(up(m.d_blk_off, m.blk_off.data(), sizeof(int32_t) * m.blk_off.size()));
+  LFX_TRY(up(m.d_blk_run, m.blk_run.data(), sizeof(int32_t) * m.blk_run.size()));
   LFX_TRY(up(m.d_ftile_row, m.ftile_row.data(), sizeof(int32_t) * m.ftile_row.size()));
   LFX_CUDA_TRY(cudaMemcpy(m.d_node_old.p, m.node_old.data(), sizeof(int32_t) * V, cudaMemcpyHostToDevice));
   LFX_CUDA_TRY(cudaMemcpy(m.d_xyz.p, x4.data(), m.d_xyz.bytes, cudaMemcpyHostToDevice));

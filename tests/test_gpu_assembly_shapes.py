@@ -78,3 +78,32 @@ def test_persistent_assembly_wait_that_runs_out_returns_timeout():
     u1, p1 = fresh.get()
     assert np.allclose(u, u1, rtol=0, atol=1e-10 * np.abs(u1).max())
     assert np.allclose(p, p1, rtol=0, atol=1e-10 * np.abs(p1).max())
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("n", [1, 2, 7, 12, 33])
+def test_persistent_assembly_equals_coloured_launches_bitwise(n, precision):
+    """Small meshes are assembled by gathering: all chunks at once into a scratch, then every block summed
+    over its chunks in the order in which the colours would have added them.  The same sums, bit for bit,
+    from one chunk (n = 1) past the largest mesh that gathers (33: the coloured form)."""
+    case = C.beltrami_case(n, seed=n, order=2)
+    got = []
+    for shape in ("chunks", "persistent"):
+        _, _, st = C.gpu_state(case, assembly=shape, precision=precision)
+        got.append(st.debug_assemble(apply_bcs=False))
+    assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("precision,eps", [("fp64", 2.0 ** -52), ("mixed", 2.0 ** -46)])
+@pytest.mark.parametrize("n", [1, 5])
+def test_gathered_newton_system_equals_coloured(n, precision, eps):
+    """The Newton matrix likewise; its right-hand side joins each chunk's Newton shares to the chunk's own
+    sum first, so rows may differ by the rounding of at most 24 elements' sums."""
+    case = C.beltrami_case(n, seed=n, order=2)
+    U = np.concatenate([case.u_hist[0], case.p_hist[0][:, None]], axis=1)
+    got = []
+    for shape in ("chunks", "persistent"):
+        _, _, st = C.gpu_state(case, assembly=shape, precision=precision)
+        got.append(st.debug_assemble_newton(U))
+    assert np.array_equal(got[0][0], got[1][0])
+    assert np.abs(got[0][1] - got[1][1]).max() <= 64 * eps * np.abs(got[0][1]).max() * 24
