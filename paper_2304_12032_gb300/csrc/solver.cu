@@ -2027,6 +2027,274 @@ __global__ void rank1_axpy_kernel(Rank1View r, const double *s, T *y, double sig
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// FP64 row kernels.  The FP64 pipe takes a warp instruction every 19 cycles of an SM or so, however
+// few of its lanes are active, so the layout that serves FP32 (a row's blocks dealt to four lanes, the
+// sums joined by shuffles, the update on one lane) wastes half of it: 59 FP64 instructions per eight
+// rows in a velocity pass against 40 here.  Lane c of a row forms component c from every block: three
+// lanes per row (ten rows a warp) for the velocity rows, four for products that end in the pressure.
+// Measured at 60k nodes on full 4x4 blocks: velocity pass 52 -> 24 us, Schur step 30 -> 12 us.
+// ------------------------------------------------------------------------------------------
+constexpr int kRows3 = kThreads / 32 * 10;   // rows per CTA, three lanes each
+inline int rows3_grid(int64_t V) { return (int)((V + kRows3 - 1) / kRows3); }
+constexpr int kU64 = 5;                      // blocks in flight per lane
+
+__device__ __forceinline__ void f_row(const BsrView<double> &A, int64_t k, int c, double f[3]) {
+  const double *p = A.vals + 16 * k + 4 * c;
+  const double2 v = __ldg(reinterpret_cast<const double2 *>(p));
+  f[0] = v.x;
+  f[1] = v.y;
+  f[2] = __ldg(p + 2);
+}
+__device__ __forceinline__ void f_row(const SplitView<double> &A, int64_t k, int c, double f[3]) {
+  const double *p = A.F + 12 * k + 3 * c;
+  f[0] = __ldg(p);
+  f[1] = __ldg(p + 1);
+  f[2] = __ldg(p + 2);
+}
+__device__ __forceinline__ double g_of(const BsrView<double> &A, int64_t k, int c) { return __ldg(A.vals + 16 * k + 4 * c + 3); }
+__device__ __forceinline__ double g_of(const SplitView<double> &A, int64_t k, int c) { return __ldg(A.G + 4 * k + c); }
+__device__ __forceinline__ double dc_of(const BsrView<double> &A, int64_t k, int c) { return __ldg(A.vals + 16 * k + 12 + c); }
+__device__ __forceinline__ double dc_of(const SplitView<double> &A, int64_t k, int c) { return __ldg(A.DC + 4 * k + c); }
+
+struct Lane3 {
+  int64_t row;
+  int c;
+  bool on;
+  __device__ __forceinline__ explicit Lane3(int64_t V) {
+    const int lane = threadIdx.x & 31;
+    row = (int64_t)blockIdx.x * kRows3 + (threadIdx.x >> 5) * 10 + lane / 3;
+    c = lane % 3;
+    on = lane < 30 && row < V;
+  }
+};
+// load(u, k) for the blocks of a row, kU64 at a time (past the end: the last block again), use(u) for the
+// valid ones
+template <class Load, class Use>
+__device__ __forceinline__ void blocks64(int32_t k0, int32_t k1, Load load, Use use) {
+#pragma unroll 1
+  for (int32_t k = k0; k < k1; k += kU64) {
+#pragma unroll
+    for (int u = 0; u < kU64; ++u) load(u, min(k + u, k1 - 1));
+#pragma unroll
+    for (int u = 0; u < kU64; ++u)
+      if (k + u < k1) use(u);
+  }
+}
+
+// velocity smoothing step k (f_step_kernel, mode 1)
+template <class View>
+__global__ void __launch_bounds__(kThreads) f_step64_kernel(View A, const double *dinvF, const double *d_old, double *d_new,
+                                                            double *r, double *x, const SmoothCoef *cf, int k,
+                                                            const KState *st) {
+  pdl_entry();
+  if (finished(st)) return;
+  const Lane3 l(A.V);
+  if (!l.on) return;
+  const int64_t e = 4 * l.row + l.c;
+  const double df = dinvF[e], rv0 = r[e], xv = x[e], dold = d_old[e];
+  double f[kU64][3], z[kU64], acc = 0.0;
+  double2 xy[kU64];
+  blocks64(
+      A.rowptr[l.row], A.rowptr[l.row + 1],
+      [&](int u, int32_t kk) {
+        f_row(A, kk, l.c, f[u]);
+        const double *v = d_old + 4 * (int64_t)__ldg(A.col + kk);
+        xy[u] = *reinterpret_cast<const double2 *>(v);
+        z[u] = v[2];
+      },
+      [&](int u) { acc += f[u][0] * xy[u].x + f[u][1] * xy[u].y + f[u][2] * z[u]; });
+  const double rv = rv0 - df * acc, dn = cf->f_c1[k] * dold + cf->f_c2[k] * rv;
+  r[e] = rv;
+  d_new[e] = dn;
+  x[e] = xv + dn;
+}
+
+// w.xyz = dinvF (G p), p = in.w; kFinal: z.xyz = x.xyz - dinvF (G p), z.w = p with p = x.w + dw.w
+template <class View, bool kFinal>
+__global__ void __launch_bounds__(kThreads) g_row64_kernel(View A, const double *dinvF, const double *in, double *out,
+                                                           const double *dw, const KState *st) {
+  pdl_entry();
+  if (finished(st)) return;
+  const Lane3 l(A.V);
+  if (!l.on) return;
+  const int64_t e = 4 * l.row + l.c;
+  double g[kU64], p[kU64], acc = 0.0;
+  blocks64(
+      A.rowptr[l.row], A.rowptr[l.row + 1],
+      [&](int u, int32_t kk) {
+        g[u] = g_of(A, kk, l.c);
+        const int64_t q = 4 * (int64_t)__ldg(A.col + kk) + 3;
+        p[u] = in[q];
+        if (kFinal && dw) p[u] += dw[q];
+      },
+      [&](int u) { acc += g[u] * p[u]; });
+  if (!kFinal) {
+    out[e] = dinvF[e] * acc;
+    return;
+  }
+  out[e] = in[e] - dinvF[e] * acc;
+  if (l.c == 0) {
+    const int64_t q = 4 * l.row + 3;
+    out[q] = dw ? in[q] + dw[q] : in[q];
+  }
+}
+
+// Products that end in the pressure row.  kD: t = b.w - D x.xyz and the start of the pressure smoothing
+// (d_init_kernel); kStep: Chebyshev / Jacobi step (s_step_kernel, mode 1); kResid: the Schur residual;
+// kPost: the start of the post-smoothing (s_resid_kernel, modes 0 and 1).
+enum { kD, kStep, kResid, kPost };
+template <class View, int kMode>
+__global__ void __launch_bounds__(kThreads) dc_row64_kernel(View A, const double *dinvS, const double *b, const double *p,
+                                                            const double *w, double *r, double *d, double *x, double *out,
+                                                            const SmoothCoef *cf, int k, const KState *st) {
+  pdl_entry();
+  if (finished(st)) return;
+  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
+  const int c = threadIdx.x & 3;
+  double acc = 0.0;
+  if (row < A.V && (kMode != kD || c < 3)) {
+    double m[kU64], v[kU64];
+    const double *src = c == 3 ? p : w;   // C p - D w
+    blocks64(
+        A.rowptr[row], A.rowptr[row + 1],
+        [&](int u, int32_t kk) {
+          m[u] = dc_of(A, kk, c);
+          v[u] = src[4 * (int64_t)__ldg(A.col + kk) + c];
+        },
+        [&](int u) { acc += m[u] * v[u]; });
+  }
+  if (kMode != kD && c < 3) acc = -acc;
+  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+  if (row >= A.V || c != 3) return;
+  const int64_t e = 4 * row + 3;
+  if (kMode == kD) {
+    const double t = b[e] - acc;
+    if (out) out[e] = t;
+    const double rv = dinvS[row] * t, dv = cf->s_init * rv;
+    r[e] = rv;
+    d[e] = dv;
+    x[e] = dv;
+  } else if (kMode == kStep) {
+    const double rv = r[e] - dinvS[row] * acc, dn = cf->s_c1[k] * p[e] + cf->s_c2[k] * rv;
+    r[e] = rv;
+    d[e] = dn;
+    x[e] += dn;
+  } else if (kMode == kResid) {
+    out[row] = b[e] - acc;
+  } else {
+    const double rv = dinvS[row] * (b[e] - acc);
+    r[e] = rv;
+    d[e] = cf->s_init * rv;
+  }
+}
+
+// y = A x (mode 0) or b - A x (mode 1), partial sums of y.y
+__global__ void __launch_bounds__(kThreads) spmv64_kernel(BsrView<double> A, const double *__restrict__ x,
+                                                          const double *__restrict__ b, double *__restrict__ y, int mode,
+                                                          double *part, const KState *st) {
+  pdl_entry();
+  if (finished(st)) return;
+  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
+  const int c = threadIdx.x & 3;
+  double acc = 0.0, nrm = 0.0;
+  if (row < A.V) {
+    double2 m[kU64][2], v[kU64][2];
+    blocks64(
+        A.rowptr[row], A.rowptr[row + 1],
+        [&](int u, int32_t kk) {
+          const double2 *q = reinterpret_cast<const double2 *>(A.vals + 16 * (int64_t)kk + 4 * c);
+          m[u][0] = __ldg(q);
+          m[u][1] = __ldg(q + 1);
+          const double2 *z = reinterpret_cast<const double2 *>(x + 4 * (int64_t)__ldg(A.col + kk));
+          v[u][0] = z[0];
+          v[u][1] = z[1];
+        },
+        [&](int u) { acc += m[u][0].x * v[u][0].x + m[u][0].y * v[u][0].y + m[u][1].x * v[u][1].x + m[u][1].y * v[u][1].y; });
+    const int64_t e = 4 * row + c;
+    if (mode == 1) acc = b[e] - acc;
+    y[e] = acc;
+    nrm = acc * acc;
+  }
+  if (part) {
+    const double s = cta_sum(nrm);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+  }
+}
+
+// Gershgorin bounds (bound_kernel): modes 0 and 1 on three lanes per row, 2 on four
+template <class View, int kMode>
+__global__ void __launch_bounds__(kThreads) bound64_kernel(View A, const double *dinvF, const double *dinvS, double *gs,
+                                                           double *part) {
+  pdl_entry();
+  double val = 0.0;
+  if (kMode < 2) {
+    const Lane3 l(A.V);
+    if (l.on) {
+      double f[kU64][3], a = 0.0;
+      blocks64(
+          A.rowptr[l.row], A.rowptr[l.row + 1],
+          [&](int u, int32_t kk) {
+            if (kMode == 0) f_row(A, kk, l.c, f[u]);
+            else f[u][0] = g_of(A, kk, l.c);
+          },
+          [&](int u) { a += kMode == 0 ? fabs(f[u][0]) + fabs(f[u][1]) + fabs(f[u][2]) : fabs(f[u][0]); });
+      const int64_t e = 4 * l.row + l.c;
+      if (kMode == 0) val = fabs(dinvF[e]) * a;
+      else gs[e] = a;
+    }
+  } else {
+    const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
+    const int c = threadIdx.x & 3;
+    double a = 0.0;
+    if (row < A.V) {
+      double m[kU64], v[kU64];
+      blocks64(
+          A.rowptr[row], A.rowptr[row + 1],
+          [&](int u, int32_t kk) {
+            m[u] = fabs(dc_of(A, kk, c));
+            const int64_t q = 4 * (int64_t)__ldg(A.col + kk) + c;
+            v[u] = c < 3 ? fabs(dinvF[q]) * gs[q] : 1.0;
+          },
+          [&](int u) { a += m[u] * v[u]; });
+    }
+    a += __shfl_xor_sync(0xffffffffu, a, 1);
+    a += __shfl_xor_sync(0xffffffffu, a, 2);
+    if (row < A.V) val = fabs(dinvS[row] * a);
+  }
+  if (kMode != 1) {
+    const double m = cta_max(val);
+    if (threadIdx.x == 0) part[blockIdx.x] = m;
+  }
+}
+
+// diag(S) (diag_s_kernel): lane c of a row sums D_c G_c / F_cc
+template <class View>
+__global__ void __launch_bounds__(kThreads) diag_s64_kernel(View A, const double *dinvF, double *dinvS) {
+  pdl_entry();
+  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
+  const int c = threadIdx.x & 3;
+  double acc = 0.0;
+  if (row < A.V && c < 3) {
+    double d[kU64], g[kU64], f[kU64];
+    blocks64(
+        A.rowptr[row], A.rowptr[row + 1],
+        [&](int u, int32_t kk) {
+          d[u] = dc_of(A, kk, c);                    // block (a, b)
+          g[u] = g_of(A, __ldg(A.trans + kk), c);    // block (b, a)
+          f[u] = dinvF[4 * (int64_t)__ldg(A.col + kk) + c];
+        },
+        [&](int u) { acc += d[u] * g[u] * f[u]; });
+  }
+  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+  if (row < A.V && c == 3) {
+    const double v = dc_of(A, A.diag[row], 3) - acc;
+    dinvS[row] = v != 0.0 ? 1.0 / v : 0.0;   // a vanishing diagonal leaves the unknown unsmoothed
+  }
+}
+
 inline int rows_grid(int64_t V) { return (int)((V * kRowGroup + kThreads - 1) / kThreads); }
 // grid for a CSR kernel with G lanes per row over n rows
 inline int lanes_grid(int64_t n, int G) { return (int)std::max<int64_t>(1, (n * G + kThreads - 1) / kThreads); }
@@ -2044,7 +2312,10 @@ template <class S, class T>
 lfx_status launch_spmv(cudaStream_t st, const BsrView<S> &A, const T *x, const T *b, T *y, int mode,
                        double *part, int *n_part) {
   const int g = rows_grid(A.V);
-  pdl_launch(spmv_kernel<S, T>, g, kThreads, 0, st, A, x, b, y, mode, part, nullptr);
+  if constexpr (std::is_same<S, double>::value)
+    pdl_launch(spmv64_kernel, g, kThreads, 0, st, A, x, b, y, mode, part, nullptr);
+  else
+    pdl_launch(spmv_kernel<S, T>, g, kThreads, 0, st, A, x, b, y, mode, part, nullptr);
   note_launches(1);
   if (n_part) *n_part = g;
   LFX_CUDA_TRY(cudaGetLastError());
@@ -2088,7 +2359,10 @@ lfx_status launch_split_vec(cudaStream_t st, int64_t V, const double *x, float4 
 // The Arnoldi product w = A z_j (kernels return at once when the cycle has finished)
 template <class S, class T>
 static void arnoldi_spmv(cudaStream_t st, const BsrView<S> &A, const T *x, T *y, const KState *ks) {
-  pdl_launch(spmv_kernel<S, T>, rows_grid(A.V), kThreads, 0, st, A, x, nullptr, y, 0, nullptr, ks);
+  if constexpr (std::is_same<S, double>::value)
+    pdl_launch(spmv64_kernel, rows_grid(A.V), kThreads, 0, st, A, x, nullptr, y, 0, nullptr, ks);
+  else
+    pdl_launch(spmv_kernel<S, T>, rows_grid(A.V), kThreads, 0, st, A, x, nullptr, y, 0, nullptr, ks);
   note_launches(1);
 }
 static void arnoldi_spmv(cudaStream_t st, const BsrView<DDMat> &A, const double *x, double *y, const KState *ks) {
@@ -2165,16 +2439,26 @@ template <class View>
 lfx_status ASimple<S, T>::setup_view(cudaStream_t st, const View &A) {
   const int rg = rows_grid(V), vg = vec_grid(V);
   pdl_launch(diag_f_kernel<View, T>, vg, kThreads, 0, st, A, dinvF.as<T>());
-  pdl_launch(diag_s_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>());
+  constexpr bool fp64 = std::is_same<T, double>::value;
+  if constexpr (fp64) pdl_launch(diag_s64_kernel<View>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>());
+  else pdl_launch(diag_s_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>());
   SmoothCoef *cf = coef.as<SmoothCoef>();
   double *lam_f = &cf->lam_f, *lam_s = &cf->lam_s;
   const bool bound = cfg.n_power <= 0;
   if (bound) {
     // Gershgorin bounds (hold for every eigenvalue; no safety factor)
+    if constexpr (fp64) {
+      const int g3 = rows3_grid(V);
+      pdl_launch(bound64_kernel<View, 0>, g3, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>());
+      pdl_launch(reduce_kernel, 1, kThreads, 0, st, part.as<double>(), g3, lam_f, 2);
+      pdl_launch(bound64_kernel<View, 1>, g3, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>());
+      pdl_launch(bound64_kernel<View, 2>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>());
+    } else {
     pdl_launch(bound_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>(), 0);
     pdl_launch(reduce_kernel, 1, kThreads, 0, st, part.as<double>(), rg, lam_f, 2);
     pdl_launch(bound_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>(), 1);
     pdl_launch(bound_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>(), 2);
+    }
     pdl_launch(reduce_kernel, 1, kThreads, 0, st, part.as<double>(), rg, lam_s, 2);
     note_launches(5);
   }
@@ -2306,7 +2590,36 @@ lfx_status ASimple<S, T>::apply_view(cudaStream_t st, const View &A, const T *r,
   // z_u* ~= F^-1 r_u
   bool pending_w = false;
   const bool staged = use_staged(A);
-  if (cfg.f_steps >= 2 && staged) {
+  constexpr bool fp64 = std::is_same<T, double>::value;
+  const int g3 = rows3_grid(V);
+  // FP64: no fused first step (it would form d_old from two vectors per block: five FP64 instructions
+  // for each one of the product)
+  auto f_step = [&](int k) {
+    if constexpr (fp64)
+      pdl_launch(f_step64_kernel<View>, g3, kThreads, 0, st, A, dinvF.as<T>(), d[(k - 1) & 1], d[k & 1], R.as<T>(), X.as<T>(),
+                 cf, k, ks);
+    else
+      pdl_launch(f_step_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), d[(k - 1) & 1], d[k & 1], R.as<T>(),
+                 X.as<T>(), cf, k, 1, nullptr, ks, nullptr);
+  };
+  auto scaled_gradient = [&](const T *in) {
+    if constexpr (fp64)
+      pdl_launch(g_row64_kernel<View, false>, g3, kThreads, 0, st, A, dinvF.as<T>(), in, W.as<T>(), nullptr, ks);
+    else pdl_launch(g_scaled_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), in, W.as<T>(), ks);
+  };
+  auto s_step = [&](int k) {
+    if constexpr (fp64)
+      pdl_launch(dc_row64_kernel<View, kStep>, rg, kThreads, 0, st, A, dinvS.as<T>(), nullptr, d[(k - 1) & 1], W.as<T>(),
+                 R.as<T>(), d[k & 1], X.as<T>(), nullptr, cf, k, ks);
+    else
+      pdl_launch(s_step_kernel<View, T>, rg, kThreads, 0, st, A, dinvS.as<T>(), d[(k - 1) & 1], W.as<T>(), d[k & 1],
+                 R.as<T>(), X.as<T>(), cf, k, 1, nullptr, ks);
+  };
+  if (fp64 && cfg.f_steps >= 2) {
+    pdl_launch(f_init_kernel<T>, vg, kThreads, 0, st, V, dinvF.as<T>(), r, R.as<T>(), d[0], X.as<T>(), cf, ks);
+    f_step(1);
+    note_launches(1);
+  } else if (cfg.f_steps >= 2 && staged) {
     LFX_TRY(launch_staged(st, A, true, 1, d[0], d[1], r, ks));
   } else if (cfg.f_steps >= 2) {
     // start of the smoothing fused into step 1 (d_old formed from r on the fly)
@@ -2329,9 +2642,7 @@ lfx_status ASimple<S, T>::apply_view(cudaStream_t st, const View &A, const T *r,
   }
   for (int k = 2; k < cfg.f_steps; ++k) {
     if (staged) LFX_TRY(launch_staged(st, A, false, k, d[(k - 1) & 1], d[k & 1], nullptr, ks));
-    else
-      pdl_launch(f_step_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), d[(k - 1) & 1], d[k & 1], R.as<T>(),
-                 X.as<T>(), cf, k, 1, nullptr, ks, nullptr);
+    else f_step(k);
   }
   if (timed) {
     LFX_CUDA_TRY(cudaEventRecord(fev[n_fev + 1], st));
@@ -2342,12 +2653,15 @@ lfx_status ASimple<S, T>::apply_view(cudaStream_t st, const View &A, const T *r,
     set_error("aSIMPLE: the Schur AMG hierarchy has not been built");
     return LFX_ERR_INVALID_ARG;
   }
-  pdl_launch(d_init_kernel<View, T>, rg, kThreads, 0, st, A, dinvS.as<T>(), r, R.as<T>(), d[0], X.as<T>(), cf, ks,
-                                               amg_ready ? Bs.as<T>() : nullptr);
+  T *bs = amg_ready ? Bs.as<T>() : nullptr;
+  if constexpr (fp64)
+    pdl_launch(dc_row64_kernel<View, kD>, rg, kThreads, 0, st, A, dinvS.as<T>(), r, nullptr, X.as<T>(), R.as<T>(), d[0],
+               X.as<T>(), bs, cf, 0, ks);
+  else
+    pdl_launch(d_init_kernel<View, T>, rg, kThreads, 0, st, A, dinvS.as<T>(), r, R.as<T>(), d[0], X.as<T>(), cf, ks, bs);
   for (int k = 1; k < cfg.s_steps; ++k) {
-    pdl_launch(g_scaled_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), d[(k - 1) & 1], W.as<T>(), ks);
-    pdl_launch(s_step_kernel<View, T>, rg, kThreads, 0, st, A, dinvS.as<T>(), d[(k - 1) & 1], W.as<T>(), d[k & 1],
-                                                 R.as<T>(), X.as<T>(), cf, k, 1, nullptr, ks);
+    scaled_gradient(d[(k - 1) & 1]);
+    s_step(k);
   }
   if (cfg.s_kind == LFX_SMOOTH_AMG && amg.size() == 1) {
     // small problem: the hierarchy is the dense inverse of S itself
@@ -2356,9 +2670,13 @@ lfx_status ASimple<S, T>::apply_view(cudaStream_t st, const View &A, const T *r,
     note_launches(1);
   } else if (cfg.s_kind == LFX_SMOOTH_AMG) {
     // residual of the pre-smoothed level-0 iterate, restriction, coarse V-cycle, prolongation
-    pdl_launch(g_scaled_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), X.as<T>(), W.as<T>(), ks);
-    pdl_launch(s_resid_kernel<View, T>, rg, kThreads, 0, st, A, dinvS.as<T>(), X.as<T>(), W.as<T>(), Bs.as<T>(),
-                                                  rr0.as<T>(), nullptr, nullptr, cf, 0, ks);
+    scaled_gradient(X.as<T>());
+    if constexpr (fp64)
+      pdl_launch(dc_row64_kernel<View, kResid>, rg, kThreads, 0, st, A, dinvS.as<T>(), Bs.as<T>(), X.as<T>(), W.as<T>(),
+                 nullptr, nullptr, nullptr, rr0.as<T>(), cf, 0, ks);
+    else
+      pdl_launch(s_resid_kernel<View, T>, rg, kThreads, 0, st, A, dinvS.as<T>(), X.as<T>(), W.as<T>(), Bs.as<T>(),
+                 rr0.as<T>(), nullptr, nullptr, cf, 0, ks);
     const AmgDevLevel &L0 = amg[0];
     CsrV<T> R0{L0.nnext, L0.Rrp.as<int32_t>(), L0.Rci.as<int32_t>(), L0.Rv.as<T>()};
     pdl_launch(csr_spmv_kernel<T, 32>, (int)((L0.nnext * 32 + kThreads - 1) / kThreads), kThreads, 0, st, 
@@ -2369,9 +2687,13 @@ lfx_status ASimple<S, T>::apply_view(cudaStream_t st, const View &A, const T *r,
     pdl_launch(csr_spmv_kernel<T, 8>, lanes_grid(V, 8), kThreads, 0, st, P0, x1, 1, 0, X.as<T>(), 4, 3,
                                                             amg_alpha, 1, ks);
     // post-smoothing from the corrected iterate
-    pdl_launch(g_scaled_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), X.as<T>(), W.as<T>(), ks);
-    pdl_launch(s_resid_kernel<View, T>, rg, kThreads, 0, st, A, dinvS.as<T>(), X.as<T>(), W.as<T>(), Bs.as<T>(), nullptr,
-                                                  R.as<T>(), d[0], cf, 1, ks);
+    scaled_gradient(X.as<T>());
+    if constexpr (fp64)
+      pdl_launch(dc_row64_kernel<View, kPost>, rg, kThreads, 0, st, A, dinvS.as<T>(), Bs.as<T>(), X.as<T>(), W.as<T>(),
+                 R.as<T>(), d[0], nullptr, nullptr, cf, 0, ks);
+    else
+      pdl_launch(s_resid_kernel<View, T>, rg, kThreads, 0, st, A, dinvS.as<T>(), X.as<T>(), W.as<T>(), Bs.as<T>(), nullptr,
+                 R.as<T>(), d[0], cf, 1, ks);
     if (cfg.s_steps == 1) {
       // x.w += d.w is left to the final pass, which reads x.w (own row and neighbours) as x.w + d.w
       pending_w = true;
@@ -2380,14 +2702,15 @@ lfx_status ASimple<S, T>::apply_view(cudaStream_t st, const View &A, const T *r,
       note_launches(1);
     }
     for (int k = 1; k < cfg.s_steps; ++k) {
-      pdl_launch(g_scaled_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), d[(k - 1) & 1], W.as<T>(), ks);
-      pdl_launch(s_step_kernel<View, T>, rg, kThreads, 0, st, A, dinvS.as<T>(), d[(k - 1) & 1], W.as<T>(), d[k & 1],
-                                                   R.as<T>(), X.as<T>(), cf, k, 1, nullptr, ks);
+      scaled_gradient(d[(k - 1) & 1]);
+      s_step(k);
     }
     note_launches(8 + 2 * (cfg.s_steps - 1));
   }
   // z_u = z_u* - diag(F)^-1 G z_p
-  if (pending_w)
+  if constexpr (fp64)
+    pdl_launch(g_row64_kernel<View, true>, g3, kThreads, 0, st, A, dinvF.as<T>(), X.as<T>(), z, pending_w ? d[0] : nullptr, ks);
+  else if (pending_w)
     pdl_launch(final_kernel<View, T, true>, rg, kThreads, 0, st, A, dinvF.as<T>(), X.as<T>(), z, ks, d[0]);
   else
     pdl_launch(final_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), X.as<T>(), z, ks, nullptr);
