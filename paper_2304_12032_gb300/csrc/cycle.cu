@@ -12,11 +12,12 @@
 // address them by 16-bit local indices (in the padding of the velocity and gradient records).  A node is read by about fifteen rows, so gathering from L2 row
 // by row moved seven times the bytes of the copy (17 us a velocity pass at 1M tetrahedra, L2-bound).
 //
-// Measured (ms per time step, before and after): 3k tetrahedra FP64 2.87 -> 1.54, 19k mixed 4.98 -> 3.28,
-// 100k FP64 15.4 -> 8.3, 150k mixed with Newton 21.3 -> 15.7, 500k mixed 16.1 -> 11.6, 600k FP64 48.4 ->
-// 33.4, 1.02M mixed 24.1 -> 19.8.  A pass costs 1.4 us for the barrier, 1.1 to 1.7 us of latency (neighbour
-// copy, records, sums) at 32 rows per CTA, and then grows with the rows: at 1M tetrahedra 14 us per velocity
-// pass and 7 us per gradient or divergence pass (L1 line lookups of the record loads), 42 us per product.
+// Measured (ms per time step, step-by-step launches and this): 3k tetrahedra FP64 2.87 and 1.54 (1.11 with
+// the gathered assembly), 19k mixed 4.98 and 3.28, 100k FP64 15.4 and 7.7, 150k mixed with Newton 21.3 and 15.7,
+// 500k mixed 16.1 and 10.9, 600k FP64 48.4 and 33.2, 1.02M mixed 24.1 and 17.9.  A pass costs 1.4 us for the
+// barrier (waiting for the halo's CTAs only: 2 us, their flags arrive one by one), 1.1 to 1.7 us of latency
+// (neighbour copy, records, sums) at 32 rows per CTA, and then grows with the rows: at 1M tetrahedra 14 us per
+// velocity pass and 7 us per gradient or divergence pass, bound by L1 line lookups of the record loads.
 // FP64 passes run at the FP64 pipe's rate (a velocity pass at 108k nodes: 45 us, 37 us of it FP64 issue).
 //
 // One extra CTA owns no rows.  It runs the FP64 recurrences of a step (Hessenberg column, rotations,
@@ -37,7 +38,7 @@ namespace lfx {
 
 namespace {
 
-constexpr int kSmemCap = 220 * 1024;
+constexpr int kSmemCap = 220 * 1024, kExtraCap = 190 * 1024;
 constexpr int kDots = 8;                  // shares of one dot product in a CTA
 
 template <class T, int LPR> struct Shape { static constexpr int threads = sizeof(T) == 8 ? 512 : 1024; };
@@ -176,6 +177,7 @@ struct Own {
   const int32_t *halo;   // [loc - n] neighbour rows of other CTAs
   int32_t loc;           // rows and halo together
   T *sv;                 // [4 (loc + 1)] the vector of the pass, then a zero entry
+  T *vb;                 // [nb][4 n] the first nb basis vectors' own rows (the others in global memory)
   T *r, *x, *df;         // [3 n] velocity residual, iterate, 1 / diag(F)
   T *t, *xp;             // [n] Schur residual, pressure iterate
   const T *ds;           // [n] 1 / diag(S)
@@ -674,7 +676,9 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
     o.halo = h;
     for (int i = threadIdx.x; i < o.loc - o.n; i += NT) h[i] = A.halo[A.halo_off[cta] + i];
   }
-  S *own_f = reinterpret_cast<S *>(sm + own_bytes(sizeof(T), A.max_rows, A.max_loc, A.spill));
+  o.vb = reinterpret_cast<T *>(sm + own_bytes(sizeof(T), A.max_rows, A.max_loc, A.spill));
+  S *own_f = reinterpret_cast<S *>(reinterpret_cast<unsigned char *>(o.vb) + A.vb_bytes);
+  const int vstride = 4 * A.max_rows, nb = (int)(A.vb_bytes / (vstride * sizeof(T)));
   const int64_t r0 = o.r0;
   // ---- the CTA's own data
   for (int i = tid; i <= o.n; i += NT) o.rp[i] = A.rowptr[r0 + i];
@@ -685,6 +689,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
     o.df[3 * i + 2] = d.z;
     if (A.spill < 1) const_cast<T *>(o.ds)[i] = A.dinvS[r0 + i];
     st4(o.w, i, v);
+    if (nb > 0) st4(o.vb, i, v);
     V4 q;
     q.x = d.x * v.x;
     q.y = d.y * v.y;
@@ -743,6 +748,8 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
     if (barrier(0)) return; \
   } while (0)
   LFX_CYCLE_SYNC();
+  const int64_t n4 = 4 * A.V;
+  auto basis = [&](int i) -> T * { return i < nb ? o.vb + (size_t)i * vstride : A.Vb + (int64_t)i * n4 + 4 * r0; };
   auto rec = [&](int row) -> const S * {
     if constexpr (fp64) return A.F + 12 * (int64_t)o.rp[row];
     return row < resident ? own_f + 12 * (int64_t)(o.rp[row] - o.rp[0]) : A.F + 12 * (int64_t)o.rp[row];
@@ -750,7 +757,6 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
   const T s0 = coef_t<T>(A.cf->f_init, A.cf->f_initf), ss0 = coef_t<T>(A.cf->s_init, A.cf->s_initf);
   T *const dbuf[2] = {A.D0, A.D1};
   const int decide_at = min(3, A.f_steps - 1);
-  const int64_t n4 = 4 * A.V;
   T s = T(1);                        // 1 / norm of the Krylov vector held in w
   unsigned long long t0 = 0, ns_f = 0, ns_p = 0;
   int j = 0, n_p = 0;
@@ -761,7 +767,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
       const T c1 = coef_t<T>(A.cf->f_c1[k], A.cf->f_c1f[k]), c2 = coef_t<T>(A.cf->f_c2[k], A.cf->f_c2f[k]);
       const T *src = first ? A.Q : dbuf[(k - 1) & 1];
       T *dst = last ? A.X : dbuf[k & 1];
-      T *vj = first && j > 0 ? A.Vb + (int64_t)j * n4 : nullptr;
+      T *vj = first && j > 0 ? basis(j) : nullptr;
       const T sa = s * s0;
       // one component: residual, step and iterate of the row
       auto update = [&](int row, int i, T a) -> T {
@@ -788,8 +794,8 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
       auto use = [&](int row, int i, T a) {
         dst[4 * (r0 + row) + i] = update(row, i, a);
         if (vj) {
-          vj[4 * (r0 + row) + i] = s * o.w[4 * row + i];
-          if (i == 0) vj[4 * (r0 + row) + 3] = s * o.w[4 * row + 3];
+          vj[4 * row + i] = s * o.w[4 * row + i];
+          if (i == 0) vj[4 * row + 3] = s * o.w[4 * row + 3];
         }
       };
       R::template velocity<S>(o, A.lcol, rec, use);
@@ -938,10 +944,10 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
       const int shares = max(1, min(kDots, NW / nv));
       for (int task = warp; task < nv * shares; task += NW) {
         const int i = task % nv, sh = task / nv;
-        const V4 *b = reinterpret_cast<const V4 *>(A.Vb + (int64_t)i * n4) + r0;
+        const V4 *b = reinterpret_cast<const V4 *>(basis(i));
         SumT a = Sm::zero();
         const int e1 = o.n * (sh + 1) / shares;
-#pragma unroll 4
+#pragma unroll (LPR == 4 ? 4 : 2)
         for (int e = o.n * sh / shares + lane; e < e1; e += 32) {
           const V4 bv = b[e], wv = ld4(o.w, e);
           Sm::add(a, bv.x * wv.x + bv.y * wv.y + bv.z * wv.z + bv.w * wv.w);
@@ -991,7 +997,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
       V4 a = ld4(o.w, e);
 #pragma unroll 4
       for (int i = 0; i < nv; ++i) {
-        const V4 b = ld4(A.Vb + (int64_t)i * n4, r0 + e);
+        const V4 b = ld4(basis(i), e);
         const T h = hs[i];
         a.x -= h * b.x;
         a.y -= h * b.y;
@@ -1111,13 +1117,16 @@ lfx_status plan_cycle(int64_t V, int64_t nnzb, const CycleMap &map, CyclePlan *p
   p->spill = sizeof(T) == 8 && own_bytes(sizeof(T), rows, map.max_loc, 0) > (size_t)kSmemCap;
   if (own_bytes(sizeof(T), rows, map.max_loc, p->spill) > (size_t)kSmemCap) return LFX_OK;
   const size_t own = own_bytes(sizeof(T), rows, map.max_loc, p->spill);
-  if (sizeof(T) == 4) {
-    // velocity records: this CTA's share with some slack, as far as they fit
-    const size_t want = (size_t)(((double)nnzb / (double)V) * 1.15 * (double)rows + 64) * 12 * sizeof(S);
-    p->f_bytes = std::min<size_t>(want, (size_t)kSmemCap - own) & ~(size_t)15;
-  }
+  // velocity records (FP32): this CTA's share with some slack, as far as they fit; then basis vectors.  Only
+  // up to kExtraCap in all: what shared memory leaves is L1, which holds the lines of the records and of the
+  // operator between a row's loads.
+  const size_t room = own < (size_t)kExtraCap ? kExtraCap - own : 0;
+  const size_t want = sizeof(T) == 4 ? (size_t)(((double)nnzb / (double)V) * 1.15 * (double)rows + 64) * 12 * sizeof(S) : 0;
+  p->f_bytes = std::min<size_t>(want, room) & ~(size_t)15;
+  const size_t vec = 4 * sizeof(T) * (size_t)rows;
+  p->vb_bytes = vec * std::min<size_t>(kMaxRestart + 1, (room - p->f_bytes) / vec);
   p->map = &map;
-  p->smem = std::max(own + p->f_bytes, kDenseSmem);
+  p->smem = std::max(own + p->vb_bytes + p->f_bytes, kDenseSmem);
   CycleKernel<S, T> k = kernel_of<S, T>(p->lanes);
   int per = 0;
   LFX_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap));
@@ -1136,6 +1145,7 @@ lfx_status launch_cycle(cudaStream_t st, const CyclePlan &p, const CycleArgs<S, 
   a.halo = p.map->halo.as<int32_t>();
   a.lcol = p.map->lcol.as<uint16_t>();
   a.f_bytes = (uint32_t)p.f_bytes;
+  a.vb_bytes = (uint32_t)p.vb_bytes;
   a.spill = p.spill;
   if (a.polls == 0) a.polls = kWaitPolls;
   LFX_CUDA_TRY(cudaMemsetAsync(a.sync, 0, offsetof(CycleSync, error), st));

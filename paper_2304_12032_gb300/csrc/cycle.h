@@ -14,6 +14,7 @@ struct CyclePlan {
   int lanes = 4;          // lanes per block row
   size_t smem = 0;
   size_t f_bytes = 0;     // of it: velocity records kept resident
+  size_t vb_bytes = 0;    // of it: basis vectors' own rows
   int spill = 0;          // row data left in global memory (own_bytes)
   int device = -1;
 };
@@ -54,7 +55,7 @@ struct CycleArgs {
   CycleSync *sync;
   int m, maxit;
   int max_rows, max_loc;
-  uint32_t f_bytes, polls;
+  uint32_t f_bytes, vb_bytes, polls;
   int spill;
 };
 

@@ -1231,12 +1231,13 @@ __global__ void div_kernel(int64_t V, const T *y, T *v, int comp_mask, const dou
 }
 
 // Chebyshev coefficients (Saad, Chebyshev acceleration) from lambda_max estimates, or the
-// constant Jacobi ones.
+// constant Jacobi ones.  Lane 0 runs the recurrence of the velocity block, lane 1 that of the Schur
+// block, then lane k converts step k (one thread doing all of it took 21 us).
 __global__ void coef_kernel(SmoothCoef *cf, int f_kind, int f_steps, double f_omega, double f_ratio,
                             int s_kind, int s_steps, double s_omega, double s_ratio, double safety) {
   pdl_entry();
-  if (threadIdx.x != 0) return;
-  for (int which = 0; which < 2; ++which) {
+  const int which = threadIdx.x;
+  if (which < 2) {
     const int kind = which ? s_kind : f_kind;
     const int steps = which ? s_steps : f_steps;
     const double omega = which ? s_omega : f_omega, ratio = which ? s_ratio : f_ratio;
@@ -1265,16 +1266,20 @@ __global__ void coef_kernel(SmoothCoef *cf, int f_kind, int f_steps, double f_om
         rho = rn;
       }
     }
-    if (which) cf->s_init = init;
-    else cf->f_init = init;
-    float *c1f = which ? cf->s_c1f : cf->f_c1f;
-    float *c2f = which ? cf->s_c2f : cf->f_c2f;
-    for (int k = 0; k < kMaxSmooth; ++k) {
-      c1f[k] = (float)c1[k];
-      c2f[k] = (float)c2[k];
+    if (which) {
+      cf->s_init = init;
+      cf->s_initf = (float)init;
+    } else {
+      cf->f_init = init;
+      cf->f_initf = (float)init;
     }
-    if (which) cf->s_initf = (float)init;
-    else cf->f_initf = (float)init;
+  }
+  __syncwarp();
+  for (int k = threadIdx.x; k < kMaxSmooth; k += 32) {
+    cf->f_c1f[k] = (float)cf->f_c1[k];
+    cf->f_c2f[k] = (float)cf->f_c2[k];
+    cf->s_c1f[k] = (float)cf->s_c1[k];
+    cf->s_c2f[k] = (float)cf->s_c2[k];
   }
 }
 
