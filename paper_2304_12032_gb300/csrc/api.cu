@@ -957,12 +957,12 @@ lfx_status lfx_problem_create(const lfx_mesh *mesh, double rho, double mu, doubl
                           cudaMemcpyHostToDevice));
   pb->asm_mode = pb->asm_mode_newton = o.assembly;
   // the row partition of the persistent Krylov cycle
-  if (o.s_smoother == LFX_SMOOTH_AMG && (m.n_comp == 1 || !o.batch_segmented)) {
+  if (o.s_smoother == LFX_SMOOTH_AMG) {
     int ctas = 0;
     const CycleMap *map = nullptr;
     if (o.precision == LFX_PREC_MIXED) LFX_TRY(cycle_ctas<float>(V, &ctas));
     else LFX_TRY(cycle_ctas<double>(V, &ctas));
-    if (ctas > 0) LFX_TRY(mesh_cycle_map(m, ctas, &map));
+    if (ctas > 0) LFX_TRY(mesh_cycle_map(m, ctas, m.n_comp > 1 && o.batch_segmented, &map));
   }
   *out = pb.release();
   return LFX_OK;
@@ -1487,7 +1487,7 @@ static lfx_status setup_asimple(lfx_state *s, ASimple<S, T> &pc) {
   lfx_problem *pb = s->pb;
   const lfx_options &o = pb->opt;
   const Mesh &m = pb->mesh->m;
-  if (m.n_comp == 1 || !o.batch_segmented) pc.plan_cycles(m);
+  pc.plan_cycles(m, m.n_comp > 1 && o.batch_segmented);
   if (s->mixed())
     LFX_TRY(pc.setup_split(s->stream, s->view<float>(s->vals32), m.nnzb));   // from the high parts
   else
@@ -1536,9 +1536,10 @@ static lfx_status run_solve(lfx_state *s, double *x, bool x_zero, int *its, int 
     auto pc = [s, A](cudaStream_t q, const double *v, double *z, const KState *ks) {
       return s->pc64.apply(q, A, v, z, ks);
     };
-    if (s->pc64.cycle_ready() && !s->gm64.segmented()) {
-      s->gm64.whole_cycle = [s, A](cudaStream_t q, double *Vb, double *Zb, double *wk, double *xx, KState *ks, int m, int maxit) {
-        return s->pc64.cycle(q, A.rowptr, A.vals, Vb, Zb, wk, xx, ks, m, maxit);
+    if (s->pc64.cycle_ready()) {
+      s->gm64.whole_cycle = [s, A](cudaStream_t q, double *Vb, double *Zb, double *wk, double *xx, KState *ks, KState *kseg,
+                                int m, int maxit) {
+        return s->pc64.cycle(q, A.rowptr, A.vals, Vb, Zb, wk, xx, ks, kseg, m, maxit);
       };
     } else {
       s->gm64.whole_cycle = nullptr;
@@ -1564,13 +1565,15 @@ static lfx_status run_solve(lfx_state *s, double *x, bool x_zero, int *its, int 
   }
   s->n_inner = 0;
   s->gm32.whole_cycle = nullptr;
-  if (async_inner && o.smoother_bf16 && s->pcbf.cycle_ready())
-    s->gm32.whole_cycle = [s, A32](cudaStream_t q, float *Vb, float *Zb, float *wk, float *xx, KState *ks, int m, int maxit) {
-      return s->pcbf.cycle(q, A32.rowptr, A32.vals, Vb, Zb, wk, xx, ks, m, maxit);
+  if (o.smoother_bf16 && s->pcbf.cycle_ready())
+    s->gm32.whole_cycle = [s, A32](cudaStream_t q, float *Vb, float *Zb, float *wk, float *xx, KState *ks, KState *kseg,
+                                int m, int maxit) {
+      return s->pcbf.cycle(q, A32.rowptr, A32.vals, Vb, Zb, wk, xx, ks, kseg, m, maxit);
     };
-  else if (async_inner && !o.smoother_bf16 && s->pc32.cycle_ready())
-    s->gm32.whole_cycle = [s, A32](cudaStream_t q, float *Vb, float *Zb, float *wk, float *xx, KState *ks, int m, int maxit) {
-      return s->pc32.cycle(q, A32.rowptr, A32.vals, Vb, Zb, wk, xx, ks, m, maxit);
+  else if (!o.smoother_bf16 && s->pc32.cycle_ready())
+    s->gm32.whole_cycle = [s, A32](cudaStream_t q, float *Vb, float *Zb, float *wk, float *xx, KState *ks, KState *kseg,
+                                int m, int maxit) {
+      return s->pc32.cycle(q, A32.rowptr, A32.vals, Vb, Zb, wk, xx, ks, kseg, m, maxit);
     };
   auto inner = [s, A32, n, &o, adaptive, async_inner](cudaStream_t q, const double *v, double *z,
                                                       const KState *ks) -> lfx_status {

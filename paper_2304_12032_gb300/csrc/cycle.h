@@ -33,6 +33,9 @@ template <class S, class T>
 struct CycleArgs {
   int64_t V;
   const int32_t *rowptr;
+  const int32_t *row_off, *cta_seg, *seg_off;   // row range and segment of each CTA, CTA range of each segment
+  int n_seg;
+  KState *kseg;                        // [n_seg] status of the segments (n_seg > 1)
   const int32_t *halo_off, *halo;      // each CTA's neighbour rows
   const uint16_t *lcol;                // [nnzb] local index of each block's column
   const S *F, *G, *DC;

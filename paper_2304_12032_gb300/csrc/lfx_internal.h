@@ -97,11 +97,12 @@ struct DBuf {
 };
 
 // ---------------------------------------------------------------- mesh (host + device)
-// The block rows dealt to `ctas` CTAs (CTA b: rows V b / ctas .. V (b + 1) / ctas), each with the list of
-// the rows of other CTAs that its blocks read (its halo, ascending), and every block's column as an index
-// into own rows followed by the halo.
+// The block rows dealt to `ctas` CTAs (consecutive ranges of nearly equal size; with segments each CTA owns
+// rows of one connected piece only), each with the list of the rows of other CTAs that its blocks read (its
+// halo, ascending), and every block's column as an index into own rows followed by the halo.
 struct CycleMap {
-  int ctas = 0, max_rows = 0, max_loc = 0;   // max_loc: largest rows + halo (columns fit 16 bits up to 65536)
+  int ctas = 0, n_seg = 1, max_rows = 0, max_loc = 0;   // max_loc: largest rows + halo (16-bit local indices)
+  DBuf row_off, cta_seg, seg_off;            // int32 [ctas + 1], [ctas], [n_seg + 1] (CTAs of a segment)
   DBuf halo_off, halo, lcol;                 // int32 [ctas + 1], int32, uint16 [nnzb]
 };
 
@@ -179,11 +180,9 @@ struct Mesh {
 lfx_status build_mesh(const double *nodes, int64_t n_nodes, const int32_t *tets, int64_t n_tets,
                       const int32_t *bfaces, const int32_t *tags, int64_t n_bfaces, Mesh &m);
 lfx_status upload_mesh(Mesh &m);
-// the mesh's map for a CTA count (host lists, uploaded); it lives as long as the mesh
-lfx_status mesh_cycle_map(const Mesh &m, int ctas, const CycleMap **out);
-// its lists: halo rows of each CTA and local column indices
-void cycle_map_lists(const Mesh &m, int ctas, std::vector<int32_t> &halo_off, std::vector<int32_t> &halo,
-                     std::vector<uint16_t> &lcol, int *max_rows, int *max_loc);
+// the mesh's map for a CTA count, with or without segments (host lists, uploaded); it lives as long as the mesh.
+// *out is null when there are more pieces than CTAs.
+lfx_status mesh_cycle_map(const Mesh &m, int ctas, bool segments, const CycleMap **out);
 
 // ---------------------------------------------------------------- kernels' parameter blocks
 constexpr int kMaxRiis = 8;

@@ -135,7 +135,7 @@ size_t Mesh::device_bytes() const {
   size_t maps = 0;
   {
     std::lock_guard<std::mutex> lk(cycle_mu);
-    for (const auto &c : cycle_maps) maps += c->halo_off.bytes + c->halo.bytes + c->lcol.bytes;
+    for (const auto &c : cycle_maps) maps += c->row_off.bytes + c->cta_seg.bytes + c->seg_off.bytes + c->halo_off.bytes + c->halo.bytes + c->lcol.bytes;
   }
   return maps + d_xyz.bytes + d_xyz_hi.bytes + d_xyz_lo.bytes + d_conn.bytes + d_slot.bytes + d_rowptr.bytes + d_col.bytes + d_diag.bytes +
          d_trans.bytes + d_comp_off.bytes + d_node_old.bytes + d_first.bytes + d_color_elems.bytes +
@@ -651,15 +651,43 @@ lfx_status upload_mesh(Mesh &m) {
   return LFX_OK;
 }
 
-void cycle_map_lists(const Mesh &m, int ctas, std::vector<int32_t> &halo_off, std::vector<int32_t> &halo,
-                     std::vector<uint16_t> &lcol, int *max_rows, int *max_loc) {
+// row ranges of the CTAs, and the CTA ranges of the segments: one more CTA at a time to the piece with the
+// most rows per CTA
+static void cycle_ranges(const Mesh &m, int ctas, bool segments, std::vector<int32_t> &row_off,
+                         std::vector<int32_t> &cta_seg, std::vector<int32_t> &seg_off) {
+  const std::vector<int32_t> all{0, (int32_t)m.V};
+  const std::vector<int32_t> &off = segments ? m.comp_off : all;
+  const int ns = (int)off.size() - 1;
+  std::vector<int> n(ns, 1);
+  for (int left = ctas - ns; left > 0; --left) {
+    int best = 0;
+    for (int c = 1; c < ns; ++c)
+      if ((int64_t)(off[c + 1] - off[c]) * n[best] > (int64_t)(off[best + 1] - off[best]) * n[c]) best = c;
+    ++n[best];
+  }
+  row_off.assign(1, 0);
+  cta_seg.clear();
+  seg_off.assign(1, 0);
+  for (int c = 0; c < ns; ++c) {
+    const int64_t rows = off[c + 1] - off[c];
+    for (int b = 0; b < n[c]; ++b) {
+      row_off.push_back(off[c] + (int32_t)(rows * (b + 1) / n[c]));
+      cta_seg.push_back(c);
+    }
+    seg_off.push_back((int32_t)cta_seg.size());
+  }
+}
+
+static void cycle_map_lists(const Mesh &m, const std::vector<int32_t> &row_off, std::vector<int32_t> &halo_off,
+                            std::vector<int32_t> &halo, std::vector<uint16_t> &lcol, int *max_rows, int *max_loc) {
+  const int ctas = (int)row_off.size() - 1;
   std::vector<std::vector<int32_t>> lists(ctas);
   lcol.assign((size_t)std::max<int64_t>(m.nnzb, 1), 0);
   const int nt = (int)std::min<unsigned>(std::max(1u, std::thread::hardware_concurrency()), 16u);
   auto work = [&](int t) {
     std::vector<int32_t> local((size_t)m.V, -1);
     for (int b = t; b < ctas; b += nt) {
-      const int32_t r0 = (int32_t)(m.V * b / ctas), r1 = (int32_t)(m.V * (b + 1) / ctas);
+      const int32_t r0 = row_off[b], r1 = row_off[b + 1];
       std::vector<int32_t> &h = lists[b];
       for (int32_t k = m.row_ptr[r0]; k < m.row_ptr[r1]; ++k) {
         const int32_t c = m.col_idx[k];
@@ -685,7 +713,7 @@ void cycle_map_lists(const Mesh &m, int ctas, std::vector<int32_t> &halo_off, st
   halo.clear();
   *max_rows = *max_loc = 0;
   for (int b = 0; b < ctas; ++b) {
-    const int rows = (int)(m.V * (b + 1) / ctas - m.V * b / ctas);
+    const int rows = row_off[b + 1] - row_off[b];
     halo.insert(halo.end(), lists[b].begin(), lists[b].end());
     halo_off.push_back((int32_t)halo.size());
     *max_rows = std::max(*max_rows, rows);
@@ -693,27 +721,35 @@ void cycle_map_lists(const Mesh &m, int ctas, std::vector<int32_t> &halo_off, st
   }
 }
 
-lfx_status mesh_cycle_map(const Mesh &m, int ctas, const CycleMap **out) {
+lfx_status mesh_cycle_map(const Mesh &m, int ctas, bool segments, const CycleMap **out) {
+  *out = nullptr;
+  const int n_seg = segments ? m.n_comp : 1;
+  if (n_seg > ctas) return LFX_OK;
   std::lock_guard<std::mutex> lk(m.cycle_mu);
   for (const auto &c : m.cycle_maps)
-    if (c->ctas == ctas) {
+    if (c->ctas == ctas && c->n_seg == n_seg) {
       *out = c.get();
       return LFX_OK;
     }
   std::unique_ptr<CycleMap> c(new (std::nothrow) CycleMap);
   if (!c) return LFX_ERR_OOM;
-  std::vector<int32_t> off, halo;
+  std::vector<int32_t> row_off, cta_seg, seg_off, off, halo;
   std::vector<uint16_t> lcol;
-  cycle_map_lists(m, ctas, off, halo, lcol, &c->max_rows, &c->max_loc);
+  cycle_ranges(m, ctas, segments, row_off, cta_seg, seg_off);
+  cycle_map_lists(m, row_off, off, halo, lcol, &c->max_rows, &c->max_loc);
   auto up = [](DBuf &d, const void *src, size_t bytes) -> lfx_status {
     LFX_TRY(d.alloc(std::max<size_t>(bytes, 16)));
     if (bytes) LFX_CUDA_TRY(cudaMemcpy(d.p, src, bytes, cudaMemcpyHostToDevice));
     return LFX_OK;
   };
+  LFX_TRY(up(c->row_off, row_off.data(), sizeof(int32_t) * row_off.size()));
+  LFX_TRY(up(c->cta_seg, cta_seg.data(), sizeof(int32_t) * cta_seg.size()));
+  LFX_TRY(up(c->seg_off, seg_off.data(), sizeof(int32_t) * seg_off.size()));
   LFX_TRY(up(c->halo_off, off.data(), sizeof(int32_t) * off.size()));
   LFX_TRY(up(c->halo, halo.data(), sizeof(int32_t) * halo.size()));
   LFX_TRY(up(c->lcol, lcol.data(), sizeof(uint16_t) * lcol.size()));
   c->ctas = ctas;
+  c->n_seg = n_seg;
   *out = c.get();
   m.cycle_maps.push_back(std::move(c));
   return LFX_OK;

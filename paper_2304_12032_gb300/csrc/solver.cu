@@ -2946,15 +2946,15 @@ lfx_status ASimple<S, T>::vcycle(cudaStream_t st, int l, const KState *ks) {
 }
 
 template <class S, class T>
-void ASimple<S, T>::plan_cycles(const Mesh &m) {
+void ASimple<S, T>::plan_cycles(const Mesh &m, bool segments) {
   int dev = 0;
   if (cfg.s_kind != LFX_SMOOTH_AMG || cfg.s_steps != 1 || cfg.f_steps < 2 || cudaGetDevice(&dev) != cudaSuccess) return;
   if (!plan) plan = new CyclePlan;
   if (plan->device == dev) return;
   int ctas = 0;
   const CycleMap *map = nullptr;
-  if (cycle_ctas<T>(V, &ctas) != LFX_OK || ctas < 1 || mesh_cycle_map(m, ctas, &map) != LFX_OK ||
-      plan_cycle<S, T>(V, m.nnzb, *map, plan) != LFX_OK) {
+  if (cycle_ctas<T>(V, &ctas) != LFX_OK || ctas < 1 || mesh_cycle_map(m, ctas, segments, &map) != LFX_OK ||
+      !map || plan_cycle<S, T>(V, m.nnzb, *map, plan) != LFX_OK) {
     *plan = CyclePlan{};   // the step-by-step path runs
     plan->device = dev;
     clear_error();
@@ -2969,7 +2969,7 @@ bool ASimple<S, T>::cycle_ready() const {
 
 template <class S, class T>
 lfx_status ASimple<S, T>::cycle(cudaStream_t st, const int32_t *rowptr, const T *A, T *Vb, T *Zb, T *wk, T *x, KState *ks,
-                                int m, int maxit) {
+                                KState *kseg, int m, int maxit) {
   if (!cyc_sync.p) {
     LFX_TRY(cyc_part.alloc(cycle_part_bytes(*plan)));
     LFX_TRY(cyc_sync.alloc(sizeof(CycleSync)));
@@ -3013,6 +3013,7 @@ lfx_status ASimple<S, T>::cycle(cudaStream_t st, const int32_t *rowptr, const T 
   a.Zb = Zb;
   a.x = x;
   a.ks = ks;
+  a.kseg = kseg;
   a.part = cyc_part.p;
   a.part_n = cyc_part.as<double>() + cycle_part_norm_offset(*plan);
   a.sync = cyc_sync.as<CycleSync>();
@@ -3339,7 +3340,9 @@ lfx_status Gmres<S, T>::solve_seg(cudaStream_t st, const BsrView<S> &A, const Pr
     pdl_launch(seg_cycle_start_kernel, 1, kThreads, 0, st, pn, tk, kseg, ks);
     pdl_launch(seg_scale_beta_kernel<T>, nt, kThreads, 0, st, w, Vb, tk, kseg);
     note_launches(3);
-    for (int j = 0; j < restart; ++j) {
+    const bool whole = whole_cycle && !cgs2;
+    if (whole) LFX_TRY(whole_cycle(st, Vb, Zb, w, x, ks, kseg, restart, maxit));
+    for (int j = 0; j < restart && !whole; ++j) {
       T *vj = Vb + (int64_t)j * n, *vn = Vb + (int64_t)(j + 1) * n, *zj = Zb + (int64_t)j * n;
       LFX_TRY(pc(st, vj, zj, ks));
       LFX_TRY(timed_spmv(st, A, zj, w, ks));
@@ -3358,9 +3361,11 @@ lfx_status Gmres<S, T>::solve_seg(cudaStream_t st, const BsrView<S> &A, const Pr
         if (pinned[(j - lag) & 3]) break;
       }
     }
-    pdl_launch(seg_trisolve_kernel, 1, kThreads, 0, st, tk, kseg);
-    pdl_launch(seg_update_x_kernel<T, T>, nt, kThreads, 0, st, Zb, n, x, tk, kseg);
-    note_launches(2);
+    if (!whole) {
+      pdl_launch(seg_trisolve_kernel, 1, kThreads, 0, st, tk, kseg);
+      pdl_launch(seg_update_x_kernel<T, T>, nt, kThreads, 0, st, Zb, n, x, tk, kseg);
+      note_launches(2);
+    }
     LFX_CUDA_TRY(cudaMemcpyAsync(&hs, ks, kStateHead, cudaMemcpyDeviceToHost, st));
     LFX_CUDA_TRY(cudaStreamSynchronize(st));
     LFX_CUDA_TRY(cudaGetLastError());
@@ -3501,7 +3506,7 @@ template <class S, class T>
 lfx_status Gmres<S, T>::run_cycle(cudaStream_t st, const BsrView<S> &A, const PrecFn<T> &pc, T *x, int m, int maxit,
                                   bool cgs2, int lag) {
   KState *ks = state.as<KState>();
-  if (whole_cycle && !cgs2 && r1.n_tags == 0) return whole_cycle(st, basis.as<T>(), zbasis.as<T>(), work.as<T>(), x, ks, m, maxit);
+  if (whole_cycle && !cgs2 && r1.n_tags == 0) return whole_cycle(st, basis.as<T>(), zbasis.as<T>(), work.as<T>(), x, ks, nullptr, m, maxit);
   LFX_TRY(arnoldi_cycle(st, A, pc, m, maxit, cgs2, lag));
   pdl_launch(trisolve_kernel, 1, 32, 0, st, ks);
   pdl_launch(update_x_kernel<T, T>, vec_grid(n), kThreads, 0, st, zbasis.as<T>(), n, x, n, ks);

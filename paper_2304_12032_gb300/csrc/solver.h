@@ -150,10 +150,10 @@ struct ASimple {
   DBuf cyc_part, cyc_sync;
   CycleSync *cyc_host = nullptr;
   void read_cycle_product(float *ms, int *count) const;   // its operator products since the last step
-  void plan_cycles(const Mesh &m);   // before setup_split, whose records carry the plan's local indices
+  void plan_cycles(const Mesh &m, bool segments);   // before setup_split, whose records carry the plan's local indices
   bool cycle_ready() const;
-  lfx_status cycle(cudaStream_t st, const int32_t *rowptr, const T *A, T *Vb, T *Zb, T *wk, T *x, KState *ks, int m,
-                   int maxit);
+  lfx_status cycle(cudaStream_t st, const int32_t *rowptr, const T *A, T *Vb, T *Zb, T *wk, T *x, KState *ks, KState *kseg,
+                   int m, int maxit);
   // Set-up on the full blocks A (the smoother then reads A's 4x4 blocks on every pass) ...
   lfx_status setup(cudaStream_t st, const BsrView<S> &A);
   // ... or on a copy of the FP64 blocks A64 converted to S with F, G and (D, C) stored apart, so
@@ -188,13 +188,13 @@ using PrecFn = std::function<lfx_status(cudaStream_t, const T *v, T *z, const KS
 template <class A, class B>
 lfx_status launch_convert(cudaStream_t st, const A *src, B *dst, int64_t n, const KState *ks);
 
-// One whole Arnoldi cycle from v_0 in Vb, the update of x included.
+// One whole Arnoldi cycle from v_0 in Vb, the update of x included (kseg: one status per segment, or null).
 template <class T>
-using CycleFn = std::function<lfx_status(cudaStream_t, T *Vb, T *Zb, T *work, T *x, KState *ks, int m, int maxit)>;
+using CycleFn = std::function<lfx_status(cudaStream_t, T *Vb, T *Zb, T *work, T *x, KState *ks, KState *kseg, int m, int maxit)>;
 
 template <class S, class T>
 struct Gmres {
-  CycleFn<T> whole_cycle;   // if set, runs a cycle of a single system (one Gram-Schmidt pass, no rank-one terms)
+  CycleFn<T> whole_cycle;   // if set, runs a cycle (one Gram-Schmidt pass, no rank-one terms)
   int64_t V = 0, n = 0;
   int restart = 40;
   int nblk_dot = 0;

@@ -51,3 +51,33 @@ def test_cycle_repeats_bit_for_bit():
         st.step()
         got.append(st.get())
     assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("precision,opts", [("fp64", {}), ("mixed", {"smoother_bf16": 1}), ("mixed", {"smoother_bf16": 0})])
+def test_cycle_of_a_batch_matches_step_by_step(precision, opts):
+    """Pieces from one smaller than a CTA's share to one over many CTAs, one at rest (a zero right-hand side
+    of its own: its solution is zero), each with its own basis, sums and stopping test."""
+    from paper_2304_12032_gb300 import lfx as L
+    from synthetic import batch, cube_kuhn
+
+    sizes = (2, 3, 9, 14)
+    m = batch([cube_kuhn(n, seed=n) for n in sizes], tag_stride=0)
+    V = m.n_nodes
+    rng = np.random.default_rng(5)
+    u0, p0 = rng.standard_normal((1, V, 3)), rng.standard_normal((1, V))
+    first = np.zeros(V, bool)
+    first[np.unique(m.tets[: 6 * sizes[0] ** 3])] = True
+    u0[0, first], p0[0, first] = 0.0, 0.0
+    bcs = [L.BC(tag=t, kind="noslip") for t in range(1, 6)] + [L.BC(tag=6, kind="neumann", time="constant", p=(0.0,))]
+    out = []
+    for reorth in (0, 2 if precision == "mixed" else 1):
+        opt = L.default_options(precision=precision, gmres_rtol=1e-11, reorthogonalize=reorth, **opts)
+        prob = L.Problem(L.Mesh.from_synthetic(m), 1.0, 0.05, 1e-2, 1, bcs, [], opt)
+        st = L.State(prob, u0, p0, 0.0)
+        stats = st.step()
+        out.append((*st.get(), stats))
+    (u, p, a), (ur, pr, b) = out
+    assert a["converged"] and b["converged"]
+    assert np.abs(u[first]).max() == 0.0 and np.abs(p[first]).max() == 0.0
+    assert rel(u, ur) < 4e-8 and rel(p, pr) < 4e-8
+    assert abs(a["iterations"] - b["iterations"]) <= 2 + b["iterations"] // 10
