@@ -181,7 +181,8 @@ struct Own {
   int32_t loc;           // rows and halo together
   T *sv;                 // [4 (loc + 1)] the vector of the pass, then a zero entry
   T *vb;                 // [nb][4 n] the first nb basis vectors' own rows (the others in global memory)
-  T *r, *x, *df;         // [3 n] velocity residual, iterate, 1 / diag(F)
+  T *r, *x;              // velocity residual and iterate, df: 1 / diag(F); three values per row, or four in
+  const T *df;           // the global vectors that take their place where shared memory is short
   T *t, *xp;             // [n] Schur residual, pressure iterate
   const T *ds;           // [n] 1 / diag(S)
   T *w;                  // [4 n] Krylov vector
@@ -517,9 +518,10 @@ struct Rows<double, LPR> {
 };
 
 // shared memory of the CTA's own data: the pass's vector, 16 values per row, halo, row pointers
-// (spill: w, t, xp and 1 / diag(S) stay in global memory)
+// (spill 1: w, t, xp and 1 / diag(S) stay in global memory, seven values per row; spill 2: r, x and 1 / diag(F)
+// too)
 __host__ __device__ inline size_t own_bytes(size_t t, int rows, int loc, int spill) {
-  const size_t n = (size_t)((rows + 3) & ~3), per = spill ? 9 : 16;
+  const size_t n = (size_t)((rows + 3) & ~3), per = spill == 0 ? 16 : (spill == 1 ? 9 : 0);
   return ((size_t)(loc + 1) * (4 * t + 4) + n * (per * t + 4) + 4 + 127) & ~(size_t)127;
 }
 
@@ -741,7 +743,8 @@ __device__ __forceinline__ void dense_algebra_seg(const CycleArgs<S, T> &A, unsi
   }
 }
 
-template <class S, class T, int LPR>
+// kFar: r, x and 1 / diag(F) in global memory (spill 2)
+template <class S, class T, int LPR, bool kFar = false>
 __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const __grid_constant__ CycleArgs<S, T> A) {
   using Sm = Sum<T>;
   using SumT = typename Sm::type;
@@ -749,6 +752,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
   using R = Rows<T, LPR>;
   constexpr int NT = Shape<T, LPR>::threads, NW = NT / 32;
   constexpr bool fp64 = sizeof(T) == 8;
+  constexpr int st = kFar ? 4 : 3;   // values per row of r, x, df
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ T hs[kMaxRestart + 1];
   __shared__ SumT red[(kMaxRestart + 1) * kDots];
@@ -774,10 +778,16 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
     T *at = reinterpret_cast<T *>(sm);
     o.sv = at;
     at += 4 * (size_t)(A.max_loc + 1);
-    o.r = at;
-    o.x = at + 3 * n;
-    o.df = at + 6 * n;
-    at += 9 * n;
+    if (!kFar) {
+      o.r = at;
+      o.x = at + 3 * n;
+      o.df = at + 6 * n;
+      at += 9 * n;
+    } else {   // W4 is free during the velocity passes; X ends up holding the iterate anyway
+      o.r = A.W4 + 4 * r;
+      o.x = A.X + 4 * r;
+      o.df = A.dinvF + 4 * r;
+    }
     if (A.spill < 1) {
       o.w = at;
       o.t = at + 4 * n;
@@ -804,9 +814,12 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
   for (int i = tid; i <= o.n; i += NT) o.rp[i] = A.rowptr[r0 + i];
   for (int i = tid; i < o.n; i += NT) {
     const V4 d = ld4(A.dinvF, r0 + i), v = ld4(A.Vb, r0 + i);
-    o.df[3 * i] = d.x;
-    o.df[3 * i + 1] = d.y;
-    o.df[3 * i + 2] = d.z;
+    if (!kFar) {
+      T *df = const_cast<T *>(o.df);
+      df[3 * i] = d.x;
+      df[3 * i + 1] = d.y;
+      df[3 * i + 2] = d.z;
+    }
     if (A.spill < 1) const_cast<T *>(o.ds)[i] = A.dinvS[r0 + i];
     st4(o.w, i, v);
     if (nb > 0) st4(o.vb, i, v);
@@ -891,7 +904,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
       const T sa = s * s0;
       // one component: residual, step and iterate of the row
       auto update = [&](int row, int i, T a) -> T {
-        const int e = 3 * row + i;
+        const int e = st * row + i;
         T rv, d0, xv;
         if (first) {
           rv = s * (o.df[e] * o.w[4 * row + i]);
@@ -955,7 +968,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
       auto scaled_gradient = [&]() {
         load1(A.xp);
         auto use = [&](int row, int i, T a) {
-          A.W4[4 * (r0 + row) + i] = o.df[3 * row + i] * a;
+          A.W4[4 * (r0 + row) + i] = o.df[st * row + i] * a;
           if (i == 0) A.W4[4 * (r0 + row) + 3] = o.xp[row];
         };
         R::gradient(o, A.G, A.lcol, use);
@@ -1044,7 +1057,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
     load1(A.pf);
     {
       auto use = [&](int row, int i, T a) {
-        zj[4 * (r0 + row) + i] = o.x[3 * row + i] - o.df[3 * row + i] * a;
+        zj[4 * (r0 + row) + i] = o.x[st * row + i] - o.df[st * row + i] * a;
         if (i == 0) zj[4 * (r0 + row) + 3] = o.sv[row];
       };
       R::gradient(o, A.G, A.lcol, use);
@@ -1124,7 +1137,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
         a.w -= h * b.w;
       }
       st4(o.w, e, a);
-      st4(A.Q, r0 + e, V4{o.df[3 * e] * a.x, o.df[3 * e + 1] * a.y, o.df[3 * e + 2] * a.z, T(0)});
+      st4(A.Q, r0 + e, V4{o.df[st * e] * a.x, o.df[st * e + 1] * a.y, o.df[st * e + 2] * a.z, T(0)});
       Sm::add(nrm, a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w);
     }
 #pragma unroll
@@ -1194,7 +1207,8 @@ constexpr int threads_of(int lanes) {
 template <class S, class T>
 using CycleKernel = void (*)(const CycleArgs<S, T>);
 template <class S, class T>
-CycleKernel<S, T> kernel_of(int lanes) {
+CycleKernel<S, T> kernel_of(int lanes, bool far) {
+  if (far) return cycle_kernel<S, T, 4, true>;
   if constexpr (sizeof(T) == 8) return lanes > 4 ? cycle_kernel<S, T, 16> : cycle_kernel<S, T, 4>;
   else return lanes > 8 ? cycle_kernel<S, T, 16> : (lanes > 4 ? cycle_kernel<S, T, 8> : cycle_kernel<S, T, 4>);
 }
@@ -1232,11 +1246,11 @@ lfx_status plan_cycle(int64_t V, int64_t nnzb, const CycleMap &map, CyclePlan *p
   p->lanes = 4;
   if (rows * 16 <= threads_of<T>(16)) p->lanes = 16;
   else if (sizeof(T) == 4 && rows * 8 <= threads_of<T>(8)) p->lanes = 8;
-  // FP64 systems keep seven of a row's sixteen values in global memory where shared memory is short (the
-  // FP64 pipe bounds their passes anyway).  FP32 systems that large (a 4M-tetrahedron stenosis, tried with
-  // all sixteen there: 113.5 against 111.6 ms a step) are bound by the matrix traffic: step by step then.
-  p->spill = sizeof(T) == 8 && own_bytes(sizeof(T), rows, map.max_loc, 0) > (size_t)kSmemCap;
-  if (own_bytes(sizeof(T), rows, map.max_loc, p->spill) > (size_t)kSmemCap) return LFX_OK;
+  // Large systems leave some or all of a row's sixteen values in global memory: 4.0M tetrahedra, 2: 95.3 ms a
+  // step against 111.6 step by step.  (Where they fit, shared memory serves them better: 1.02M, 0: 18.0 ms, 1: 18.5.)
+  for (p->spill = 0; p->spill <= 2; ++p->spill)
+    if (own_bytes(sizeof(T), rows, map.max_loc, p->spill) <= (size_t)kSmemCap) break;
+  if (p->spill > 2) return LFX_OK;
   const size_t own = own_bytes(sizeof(T), rows, map.max_loc, p->spill);
   // velocity records (FP32): this CTA's share with some slack, as far as they fit; then basis vectors.  Only
   // up to kExtraCap in all: what shared memory leaves is L1, which holds the lines of the records and of the
@@ -1248,7 +1262,7 @@ lfx_status plan_cycle(int64_t V, int64_t nnzb, const CycleMap &map, CyclePlan *p
   p->vb_bytes = vec * std::min<size_t>(kMaxRestart + 1, (room - p->f_bytes) / vec);
   p->map = &map;
   p->smem = std::max(own + p->vb_bytes + p->f_bytes, kDenseSmem);
-  CycleKernel<S, T> k = kernel_of<S, T>(p->lanes);
+  CycleKernel<S, T> k = kernel_of<S, T>(p->lanes, p->spill == 2);
   int per = 0;
   LFX_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemCap));
   LFX_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, threads_of<T>(p->lanes), p->smem));
@@ -1275,7 +1289,7 @@ lfx_status launch_cycle(cudaStream_t st, const CyclePlan &p, const CycleArgs<S, 
   if (a.polls == 0) a.polls = kWaitPolls;
   LFX_CUDA_TRY(cudaMemsetAsync(a.sync, 0, offsetof(CycleSync, error), st));
   void *kargs[] = {&a};
-  LFX_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)kernel_of<S, T>(p.lanes), dim3(p.rows_ctas + 1),
+  LFX_CUDA_TRY(cudaLaunchCooperativeKernel((const void *)kernel_of<S, T>(p.lanes, p.spill == 2), dim3(p.rows_ctas + 1),
                                            dim3(threads_of<T>(p.lanes)), kargs, p.smem, st));
   note_launches(1);
   return LFX_OK;
