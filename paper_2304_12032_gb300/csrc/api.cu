@@ -1713,6 +1713,23 @@ static lfx_status newton_residual_norm(lfx_state *s, double *out) {
   return LFX_OK;
 }
 
+// The status of a solve that ended with `rc`: LFX_ERR_TIMEOUT if one of its bounded waits gave up.
+// A hard error can be the trace of such a wait (values that were never written), and a flag left
+// set would be reported by the next step.
+static lfx_status waits_checked(lfx_state *s, lfx_status rc, const char *who) {
+  if (rc == LFX_ERR_CUDA) return rc;
+  cudaStream_t st = s->stream;
+  if (!s->mixed()) LFX_TRY(s->pc64.queue_bulk_check(st));
+  else if (s->pb->opt.smoother_bf16) LFX_TRY(s->pcbf.queue_bulk_check(st));
+  else LFX_TRY(s->pc32.queue_bulk_check(st));
+  LFX_CUDA_TRY(cudaStreamSynchronize(st));
+  if (!(s->pcbf.bulk_failed() | s->pc32.bulk_failed() | s->pc64.bulk_failed())) return rc;
+  s->assembled = false;
+  set_error("%s: a bounded wait of the linear solve (a staged tile of the velocity smoothing pass, or a "
+            "grid-wide wait of the persistent Krylov cycle) gave up; the state was not advanced", who);
+  return LFX_ERR_TIMEOUT;
+}
+
 // Newton iterations of the fully implicit formulation (Section 2.4) from the semi-implicit solution
 // in xsol: stop once ||R(U_k)|| <= newton_rtol * scale, else assemble J(U_k) and b + X U_k and solve
 // J U_{k+1} = b + X U_k from U_k.
@@ -1912,14 +1929,14 @@ lfx_status lfx_step(lfx_state *s, lfx_step_stats *stats) {
   s->pc32.n_fev = 0;
   s->pcbf.n_fev = 0;
   lfx_status rc = run_solve(s, s->xsol.as<double>(), false, &its, &outer, &rel);
-  if (rc != LFX_OK && rc != LFX_ERR_NOT_CONVERGED) return rc;
+  if (rc != LFX_OK && rc != LFX_ERR_NOT_CONVERGED) return waits_checked(s, rc, "lfx_step");
   int n_newton = 0;
   float ms_newton = 0.0f, ms_asm_semi = 0.0f;
   if (o.implicit) {
     LFX_CUDA_TRY(cudaEventSynchronize(s->ea1));
     cudaEventElapsedTime(&ms_asm_semi, s->ea0, s->ea1);
     lfx_status rn = newton_loop(s, scale, &n_newton, &its, &outer, &rel, &ms_newton);
-    if (rn != LFX_OK && rn != LFX_ERR_NOT_CONVERGED) return rn;
+    if (rn != LFX_OK && rn != LFX_ERR_NOT_CONVERGED) return waits_checked(s, rn, "lfx_step");
     if (rn == LFX_ERR_NOT_CONVERGED) rc = rn;
   } else {
     s->newton_res.clear();
@@ -1937,7 +1954,7 @@ lfx_status lfx_step(lfx_state *s, lfx_step_stats *stats) {
     set_error("lfx_step: a grid-wide wait of the persistent assembly gave up; the state was not advanced");
     return LFX_ERR_TIMEOUT;
   }
-  if (s->pcbf.bulk_failed() || s->pc32.bulk_failed() || s->pc64.bulk_failed()) {
+  if (s->pcbf.bulk_failed() | s->pc32.bulk_failed() | s->pc64.bulk_failed()) {
     set_error("lfx_step: a bounded wait of the linear solve (a staged tile of the velocity smoothing pass, or a "
               "grid-wide wait of the persistent Krylov cycle) gave up; the state was not advanced");
     return LFX_ERR_TIMEOUT;
@@ -2301,6 +2318,8 @@ lfx_status lfx_debug_solve(lfx_state *s, double *x, lfx_step_stats *stats) {
   int its = 0, outer = 0;
   double rel = 0;
   lfx_status rc = run_solve(s, dx.as<double>(), true, &its, &outer, &rel);
+  rc = waits_checked(s, rc, "lfx_debug_solve");
+  if (rc == LFX_ERR_TIMEOUT) return rc;
   if (stats) {
     memset(stats, 0, sizeof(*stats));
     stats->iterations = its;
