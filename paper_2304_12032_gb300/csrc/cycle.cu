@@ -756,7 +756,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ T hs[kMaxRestart + 1];
   __shared__ SumT red[(kMaxRestart + 1) * kDots];
-  __shared__ int verdict, resident;
+  __shared__ int verdict, resident, solved;
   if (finished(A.ks) || *(volatile const int *)&A.sync->error) return;
   const unsigned rows_ctas = gridDim.x - 1, cta = blockIdx.x;
   if (cta == rows_ctas) {
@@ -1166,12 +1166,13 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
   }
 ended:
   // ---- x += sum_i y_i z_i over the steps taken (j of them)
+  // (a word of its own: other warps may still be reading the verdict that sent them here)
   if (tid == 0) {
-    verdict = wait_for(&A.sync->solved, 1u, A.polls) ? 0 : 1;
-    if (verdict) atomicExch(&A.sync->error, 1);
+    solved = wait_for(&A.sync->solved, 1u, A.polls);
+    if (!solved) atomicExch(&A.sync->error, 1);
   }
   __syncthreads();
-  if (verdict) return;
+  if (!solved) return;
   const KState *own = A.n_seg > 1 ? A.kseg + A.cta_seg[cta] : A.ks;
   if (A.n_seg > 1) j = own->j;   // (steps until this segment had converged)
   for (int i = tid; i < j; i += NT) hs[i] = (T)own->y[i];
