@@ -398,6 +398,10 @@ lfx_status lfx_debug_persistent_timeout(lfx_state *state);
  * returns.  LFX_ERR_TIMEOUT is the expected result; the state stays usable (the next lfx_step
  * assembles anew).  Needs a mixed-precision state with smoother_bf16 and staged_f set. */
 lfx_status lfx_debug_staged_timeout(lfx_state *state);
+/* on = 1: from now on the grid-wide waits of the state's persistent Krylov cycles get a target that
+ * nothing reaches and a limit of milliseconds, so that they run out (LFX_ERR_TIMEOUT from lfx_step);
+ * on = 0: back to normal.  Host-only. */
+lfx_status lfx_debug_cycle_timeout(lfx_state *state, int32_t on);
 /* y = A x with the last assembled matrix; x, y [n_nodes][4] FP64 host buffers, caller numbering. */
 lfx_status lfx_debug_spmv(lfx_state *state, const double *x, double *y);
 /* z = P^-1 r with the aSIMPLE preconditioner of the last assembled matrix (FP64 path);

@@ -1538,8 +1538,8 @@ static lfx_status run_solve(lfx_state *s, double *x, bool x_zero, int *its, int 
     };
     if (s->pc64.cycle_ready()) {
       s->gm64.whole_cycle = [s, A](cudaStream_t q, double *Vb, double *Zb, double *wk, double *xx, KState *ks, KState *kseg,
-                                int m, int maxit) {
-        return s->pc64.cycle(q, A.rowptr, A.vals, Vb, Zb, wk, xx, ks, kseg, m, maxit);
+                                KState *parent, int m, int maxit) {
+        return s->pc64.cycle(q, A.rowptr, A.vals, Vb, Zb, wk, xx, ks, kseg, parent, m, maxit);
       };
     } else {
       s->gm64.whole_cycle = nullptr;
@@ -1567,16 +1567,17 @@ static lfx_status run_solve(lfx_state *s, double *x, bool x_zero, int *its, int 
   s->gm32.whole_cycle = nullptr;
   if (o.smoother_bf16 && s->pcbf.cycle_ready())
     s->gm32.whole_cycle = [s, A32](cudaStream_t q, float *Vb, float *Zb, float *wk, float *xx, KState *ks, KState *kseg,
-                                int m, int maxit) {
-      return s->pcbf.cycle(q, A32.rowptr, A32.vals, Vb, Zb, wk, xx, ks, kseg, m, maxit);
+                                KState *parent, int m, int maxit) {
+      return s->pcbf.cycle(q, A32.rowptr, A32.vals, Vb, Zb, wk, xx, ks, kseg, parent, m, maxit);
     };
   else if (!o.smoother_bf16 && s->pc32.cycle_ready())
     s->gm32.whole_cycle = [s, A32](cudaStream_t q, float *Vb, float *Zb, float *wk, float *xx, KState *ks, KState *kseg,
-                                int m, int maxit) {
-      return s->pc32.cycle(q, A32.rowptr, A32.vals, Vb, Zb, wk, xx, ks, kseg, m, maxit);
+                                KState *parent, int m, int maxit) {
+      return s->pc32.cycle(q, A32.rowptr, A32.vals, Vb, Zb, wk, xx, ks, kseg, parent, m, maxit);
     };
   auto inner = [s, A32, n, &o, adaptive, async_inner](cudaStream_t q, const double *v, double *z,
                                                       const KState *ks) -> lfx_status {
+    s->gm32.parent = const_cast<KState *>(ks);
     LFX_TRY((launch_convert<double, float>(q, v, s->r32.as<float>(), n, ks)));
     if (async_inner) {
       int *slot = s->inner_its + std::min(s->n_inner, s->inner_cap - 1);
@@ -2140,6 +2141,16 @@ lfx_status lfx_debug_staged_timeout(lfx_state *s) {
     set_error("staged velocity smoothing pass: a wait for a tile gave up");
     return LFX_ERR_TIMEOUT;
   }
+  return LFX_OK;
+}
+
+lfx_status lfx_debug_cycle_timeout(lfx_state *s, int32_t on) {
+  clear_error();
+  if (!s) {
+    set_error("lfx_debug_cycle_timeout: NULL state");
+    return LFX_ERR_INVALID_ARG;
+  }
+  s->pc64.force_cycle_timeout = s->pc32.force_cycle_timeout = s->pcbf.force_cycle_timeout = on != 0;
   return LFX_OK;
 }
 

@@ -28,7 +28,8 @@
 // and they read its verdict after the first of those passes.
 //
 // Every wait is bounded: a CTA that gives up sets the error word and returns, the others then run into
-// their own limits; the host reports LFX_ERR_TIMEOUT.
+// their own limits.  The CTA without rows, or the next cycle's at its start, flags the solve's status, and the
+// host ends the solve with LFX_ERR_TIMEOUT.
 #include <algorithm>
 #include <cstddef>
 #include <type_traits>
@@ -530,6 +531,19 @@ __host__ __device__ inline int step_barriers(int f_steps, int L, bool fp64) {
   return (f_steps - 1) + 1 + (L == 1 ? 1 : 7 + 4 * (L - 2)) + 1 + (fp64 ? 3 : 2);
 }
 
+// one thread of the CTA without rows: a wait ran out, which ends the solve and the one that it preconditions
+// (the host reads the flag with the status of the cycle)
+template <class S, class T>
+__device__ __forceinline__ void gave_up(const CycleArgs<S, T> &A) {
+  atomicExch(&A.sync->error, 1);
+  A.ks->flag = kFlagTimeout;
+  A.ks->done = 1;
+  if (A.parent) {
+    A.parent->flag = kFlagTimeout;
+    A.parent->done = 1;
+  }
+}
+
 // The CTA without rows: Hessenberg columns, rotations, stopping test, back substitution (FP64).
 template <class S, class T, int LPR>
 __device__ __forceinline__ void dense_algebra(const CycleArgs<S, T> &A, unsigned char *sm, unsigned rows_ctas) {
@@ -548,9 +562,9 @@ __device__ __forceinline__ void dense_algebra(const CycleArgs<S, T> &A, unsigned
   if (threadIdx.x == 0) g[0] = ks->g[0];
   auto reached = [&](unsigned barriers) {
     __syncthreads();
-    if (threadIdx.x == 0) go = wait_for(&A.sync->arrived, barriers * rows_ctas, A.polls);
+    if (threadIdx.x == 0) go = wait_for(&A.sync->arrived, barriers * rows_ctas + A.unreachable, A.polls);
     __syncthreads();
-    if (!go && threadIdx.x == 0) atomicExch(&A.sync->error, 1);
+    if (!go && threadIdx.x == 0) gave_up(A);
     return go != 0;
   };
   for (int j = 0;; ++j) {
@@ -646,9 +660,9 @@ __device__ __forceinline__ void dense_algebra_seg(const CycleArgs<S, T> &A, unsi
   int total = A.ks->total;
   auto reached = [&](unsigned barriers) {
     __syncthreads();
-    if (threadIdx.x == 0) go = wait_for(&A.sync->arrived, barriers * rows_ctas, A.polls);
+    if (threadIdx.x == 0) go = wait_for(&A.sync->arrived, barriers * rows_ctas + A.unreachable, A.polls);
     __syncthreads();
-    if (!go && threadIdx.x == 0) atomicExch(&A.sync->error, 1);
+    if (!go && threadIdx.x == 0) gave_up(A);
     return go != 0;
   };
   for (int j = 0;; ++j) {
@@ -757,8 +771,12 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
   __shared__ T hs[kMaxRestart + 1];
   __shared__ SumT red[(kMaxRestart + 1) * kDots];
   __shared__ int verdict, resident, solved;
-  if (finished(A.ks) || *(volatile const int *)&A.sync->error) return;
+  if (finished(A.ks)) return;
   const unsigned rows_ctas = gridDim.x - 1, cta = blockIdx.x;
+  if (*(volatile const int *)&A.sync->error) {   // a wait of an earlier cycle gave up
+    if (cta == rows_ctas && threadIdx.x == 0) gave_up(A);
+    return;
+  }
   if (cta == rows_ctas) {
     if (A.n_seg > 1) dense_algebra_seg<S, T, LPR>(A, rows_ctas);
     else dense_algebra<S, T, LPR>(A, sm, rows_ctas);
@@ -865,7 +883,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
     target += rows_ctas;
     if (tid == 0) {
       arrive(&A.sync->arrived);
-      int v = wait_for(&A.sync->arrived, target, A.polls) ? 0 : 1;
+      int v = wait_for(&A.sync->arrived, target + A.unreachable, A.polls) ? 0 : 1;
       if (v == 0 && decide > 0) {
         if (!wait_for(&A.sync->progress, 2u * (unsigned)decide, A.polls)) v = 1;
         else if (ld_relaxed(&A.sync->progress) & 1u) v = 2;

@@ -53,12 +53,13 @@ struct CycleArgs {
   const T *x1, *coarse_inv;
   T alpha;
   T *Vb, *Zb, *x;
-  KState *ks;
+  KState *ks, *parent;                 // status; that of the flexible solve it preconditions, or null
   void *part, *part_n;                 // [kMaxRestart + 1][rows_ctas], [rows_ctas] partial sums
   CycleSync *sync;
   int m, maxit;
   int max_rows, max_loc;
-  uint32_t f_bytes, vb_bytes, polls;
+  uint32_t f_bytes, vb_bytes, polls;   // polls: limit of every wait (0: kWaitPolls)
+  unsigned unreachable;                // added to the arrivals that a barrier waits for (tests: it gives up)
   int spill;
 };
 

@@ -7,6 +7,7 @@
 namespace lfx {
 
 constexpr uint32_t kWaitPolls = 1u << 22;   // seconds of polls; a wait that runs out gives up
+constexpr uint32_t kTestPolls = 1u << 12;   // milliseconds: the limit of waits that a test makes run out
 
 __device__ __forceinline__ unsigned ld_relaxed(const unsigned *p) {
   unsigned v;

@@ -21,6 +21,7 @@
 #include "amg.h"
 #include "cycle.h"
 #include "dd.h"
+#include "grid_wait.h"
 #include "kernels.h"
 #include "pdl.h"
 #include "solver.h"
@@ -2969,7 +2970,7 @@ bool ASimple<S, T>::cycle_ready() const {
 
 template <class S, class T>
 lfx_status ASimple<S, T>::cycle(cudaStream_t st, const int32_t *rowptr, const T *A, T *Vb, T *Zb, T *wk, T *x, KState *ks,
-                                KState *kseg, int m, int maxit) {
+                                KState *kseg, KState *parent, int m, int maxit) {
   if (!cyc_sync.p) {
     LFX_TRY(cyc_part.alloc(cycle_part_bytes(*plan)));
     LFX_TRY(cyc_sync.alloc(sizeof(CycleSync)));
@@ -3014,11 +3015,16 @@ lfx_status ASimple<S, T>::cycle(cudaStream_t st, const int32_t *rowptr, const T 
   a.x = x;
   a.ks = ks;
   a.kseg = kseg;
+  a.parent = parent;
   a.part = cyc_part.p;
   a.part_n = cyc_part.as<double>() + cycle_part_norm_offset(*plan);
   a.sync = cyc_sync.as<CycleSync>();
   a.m = m;
   a.maxit = maxit;
+  if (force_cycle_timeout) {
+    a.unreachable = 1;
+    a.polls = kTestPolls;
+  }
   return launch_cycle<S, T>(st, *plan, a);
 }
 
@@ -3202,6 +3208,11 @@ lfx_status Gmres<S, T>::solve(cudaStream_t st, const BsrView<S> &A, const PrecFn
       status = LFX_OK;
       break;
     }
+    if (hs.flag == kFlagTimeout) {
+      set_error("GMRES: a grid-wide wait of the persistent cycle gave up after %d steps", total);
+      status = LFX_ERR_TIMEOUT;
+      break;
+    }
     if (hs.flag == 2) {
       set_error("GMRES: non-finite residual after %d steps", total);
       status = LFX_ERR_NONFINITE;
@@ -3341,7 +3352,7 @@ lfx_status Gmres<S, T>::solve_seg(cudaStream_t st, const BsrView<S> &A, const Pr
     pdl_launch(seg_scale_beta_kernel<T>, nt, kThreads, 0, st, w, Vb, tk, kseg);
     note_launches(3);
     const bool whole = whole_cycle && !cgs2;
-    if (whole) LFX_TRY(whole_cycle(st, Vb, Zb, w, x, ks, kseg, restart, maxit));
+    if (whole) LFX_TRY(whole_cycle(st, Vb, Zb, w, x, ks, kseg, parent, restart, maxit));
     for (int j = 0; j < restart && !whole; ++j) {
       T *vj = Vb + (int64_t)j * n, *vn = Vb + (int64_t)(j + 1) * n, *zj = Zb + (int64_t)j * n;
       LFX_TRY(pc(st, vj, zj, ks));
@@ -3370,6 +3381,11 @@ lfx_status Gmres<S, T>::solve_seg(cudaStream_t st, const BsrView<S> &A, const Pr
     LFX_CUDA_TRY(cudaStreamSynchronize(st));
     LFX_CUDA_TRY(cudaGetLastError());
     total = hs.total;
+    if (hs.flag == kFlagTimeout) {
+      set_error("GMRES: a grid-wide wait of the persistent cycle gave up after %d steps", total);
+      status = LFX_ERR_TIMEOUT;
+      break;
+    }
     if (hs.flag == 2) {
       set_error("GMRES: non-finite residual after %d steps", total);
       status = LFX_ERR_NONFINITE;
@@ -3506,7 +3522,8 @@ template <class S, class T>
 lfx_status Gmres<S, T>::run_cycle(cudaStream_t st, const BsrView<S> &A, const PrecFn<T> &pc, T *x, int m, int maxit,
                                   bool cgs2, int lag) {
   KState *ks = state.as<KState>();
-  if (whole_cycle && !cgs2 && r1.n_tags == 0) return whole_cycle(st, basis.as<T>(), zbasis.as<T>(), work.as<T>(), x, ks, nullptr, m, maxit);
+  if (whole_cycle && !cgs2 && r1.n_tags == 0)
+    return whole_cycle(st, basis.as<T>(), zbasis.as<T>(), work.as<T>(), x, ks, nullptr, parent, m, maxit);
   LFX_TRY(arnoldi_cycle(st, A, pc, m, maxit, cgs2, lag));
   pdl_launch(trisolve_kernel, 1, 32, 0, st, ks);
   pdl_launch(update_x_kernel<T, T>, vec_grid(n), kThreads, 0, st, zbasis.as<T>(), n, x, n, ks);

@@ -13,6 +13,7 @@ namespace lfx {
 
 constexpr int kMaxRestart = 64;
 constexpr int kMaxSmooth = 32;
+constexpr int kFlagTimeout = 3;   // KState::flag of a solve whose persistent cycle's wait gave up
 
 struct SmootherConfig {
   int f_kind = LFX_SMOOTH_CHEBYSHEV, f_steps = 3;
@@ -40,7 +41,7 @@ struct KState {
   int done;                       // cycle finished (converged, full, or failed)
   int j;                          // Arnoldi steps completed in this cycle
   int total;                      // steps over all cycles
-  int flag;                       // 0 running/full, 1 converged, 2 non-finite
+  int flag;                       // 0 running/full, 1 converged, 2 non-finite, kFlagTimeout: a wait gave up
   double bnorm, tol_abs, beta, res, scale;
   double H[kMaxRestart * (kMaxRestart + 1)];   // column-major, ld = kMaxRestart + 1
   double g[kMaxRestart + 1], cs[kMaxRestart], sn[kMaxRestart], y[kMaxRestart];
@@ -149,11 +150,12 @@ struct ASimple {
   CyclePlan *plan = nullptr;
   DBuf cyc_part, cyc_sync;
   CycleSync *cyc_host = nullptr;
+  bool force_cycle_timeout = false;   // tests: the cycles' grid-wide waits run out
   void read_cycle_product(float *ms, int *count) const;   // its operator products since the last step
   void plan_cycles(const Mesh &m, bool segments);   // before setup_split, whose records carry the plan's local indices
   bool cycle_ready() const;
   lfx_status cycle(cudaStream_t st, const int32_t *rowptr, const T *A, T *Vb, T *Zb, T *wk, T *x, KState *ks, KState *kseg,
-                   int m, int maxit);
+                   KState *parent, int m, int maxit);
   // Set-up on the full blocks A (the smoother then reads A's 4x4 blocks on every pass) ...
   lfx_status setup(cudaStream_t st, const BsrView<S> &A);
   // ... or on a copy of the FP64 blocks A64 converted to S with F, G and (D, C) stored apart, so
@@ -188,13 +190,16 @@ using PrecFn = std::function<lfx_status(cudaStream_t, const T *v, T *z, const KS
 template <class A, class B>
 lfx_status launch_convert(cudaStream_t st, const A *src, B *dst, int64_t n, const KState *ks);
 
-// One whole Arnoldi cycle from v_0 in Vb, the update of x included (kseg: one status per segment, or null).
+// One whole Arnoldi cycle from v_0 in Vb, the update of x included (kseg: one status per segment, or null;
+// parent: Gmres::parent).
 template <class T>
-using CycleFn = std::function<lfx_status(cudaStream_t, T *Vb, T *Zb, T *work, T *x, KState *ks, KState *kseg, int m, int maxit)>;
+using CycleFn = std::function<lfx_status(cudaStream_t, T *Vb, T *Zb, T *work, T *x, KState *ks, KState *kseg,
+                                          KState *parent, int m, int maxit)>;
 
 template <class S, class T>
 struct Gmres {
   CycleFn<T> whole_cycle;   // if set, runs a cycle (one Gram-Schmidt pass, no rank-one terms)
+  KState *parent = nullptr;   // status of the flexible solve that this one preconditions: a wait that gives up ends both
   int64_t V = 0, n = 0;
   int restart = 40;
   int nblk_dot = 0;

@@ -133,6 +133,7 @@ _SIGS = {
     "lfx_debug_assemble_newton": ([_P, _DP, _DP, _DP], ctypes.c_int32),
     "lfx_debug_persistent_timeout": ([_P], ctypes.c_int32),
     "lfx_debug_staged_timeout": ([_P], ctypes.c_int32),
+    "lfx_debug_cycle_timeout": ([_P, ctypes.c_int32], ctypes.c_int32),
     "lfx_debug_precond": ([_P, _DP, _DP, _DP, _DP], ctypes.c_int32),
     "lfx_debug_solve": ([_P, _DP, ctypes.POINTER(lfx_step_stats)], ctypes.c_int32),
     "lfx_set_allocator": ([ALLOC_FN, FREE_FN, _P], ctypes.c_int32),
@@ -548,6 +549,10 @@ class State:
     def debug_staged_timeout(self):
         """Status of one BF16 preconditioner application whose staged-tile waits are made to run out."""
         return library().lfx_debug_staged_timeout(self.h)
+
+    def debug_cycle_timeout(self, on):
+        """Make the grid-wide waits of the persistent Krylov cycles run out from now on, or not any more."""
+        _check(library().lfx_debug_cycle_timeout(self.h, int(on)))
 
     def debug_spmv(self, x):
         x = np.ascontiguousarray(x, dtype=np.float64).reshape(self.V, 4)
