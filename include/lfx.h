@@ -402,6 +402,8 @@ lfx_status lfx_debug_staged_timeout(lfx_state *state);
  * nothing reaches and a limit of milliseconds, so that they run out (LFX_ERR_TIMEOUT from lfx_step);
  * on = 0: back to normal.  Host-only. */
 lfx_status lfx_debug_cycle_timeout(lfx_state *state, int32_t on);
+/* The same for the grid-wide waits of a moving mesh's lifting. */
+lfx_status lfx_debug_lifting_timeout(lfx_state *state, int32_t on);
 /* y = A x with the last assembled matrix; x, y [n_nodes][4] FP64 host buffers, caller numbering. */
 lfx_status lfx_debug_spmv(lfx_state *state, const double *x, double *y);
 /* z = P^-1 r with the aSIMPLE preconditioner of the last assembled matrix (FP64 path);

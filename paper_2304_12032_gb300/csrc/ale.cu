@@ -247,6 +247,8 @@ struct CgArgs {
   double tol2;
   int max_iters, max_rows;
   uint32_t k_entries;     // matrix entries that fit beside the vectors
+  uint32_t polls;         // limit of every grid-wide wait
+  unsigned unreachable;   // added to the arrivals that a wait needs (tests: it gives up)
 };
 
 __host__ __device__ inline size_t cg_own_bytes(int rows) {
@@ -290,7 +292,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) lifting_cg_kernel(const __grid_
     target += ctas;
     if (tid == 0) {
       arrive(&A.cs->arrived);
-      ok = wait_for(&A.cs->arrived, target, kWaitPolls);
+      ok = wait_for(&A.cs->arrived, target + A.unreachable, A.polls);
       if (!ok) atomicExch(&A.cs->error, 1);
     }
     __syncthreads();
@@ -508,7 +510,8 @@ lfx_status lifting_solve(cudaStream_t st, const LiftingView &L, int64_t n_fixed,
   const int ctas = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)sms, (int64_t)kCgMaxCtas, V / kCgMinRows}));
   const int rows = (int)((V + ctas - 1) / ctas);
   if (coop && cg_own_bytes(rows) <= (size_t)kCgSmem) {
-    CgArgs A{V, L.rowptr, L.col, L.K, L.dinv, L.fixed, d, L.p, L.part, cs, rtol * rtol, max_iters, rows, 0};
+    CgArgs A{V, L.rowptr, L.col, L.K, L.dinv, L.fixed, d, L.p, L.part, cs, rtol * rtol, max_iters, rows, 0,
+             L.force_timeout ? kTestPolls : kWaitPolls, L.force_timeout ? 1u : 0u};
     const size_t own = cg_own_bytes(rows), entry = sizeof(double) + sizeof(int32_t);
     A.k_entries = (uint32_t)(((size_t)kCgSmem - own) / entry) & ~1u;
     A.k_entries = std::min<uint32_t>(A.k_entries, (uint32_t)std::min<int64_t>(40LL * rows, 1 << 20));

@@ -204,6 +204,7 @@ struct lfx_state {
   int *asm_err_host = nullptr;
   int asm_mode_used = 0;
   bool force_timeout = false;   // tests: make the persistent assembly's first grid-wide wait run out
+  bool force_lifting_timeout = false;   // tests: likewise the lifting's
   int64_t n_bnd = 0;
   D4 *dlevel(int l) { return dhist[(dhead + l) % sigma].as<D4>(); }
   ~lfx_state() {
@@ -1651,7 +1652,7 @@ static lfx_status ale_prepare(lfx_state *s) {
   LFX_CUDA_TRY(cudaMemcpyAsync(s->dnew.p, s->dlevel(0), sizeof(D4) * (size_t)V, cudaMemcpyDeviceToDevice, st));
   const LiftingView L{V, m.d_rowptr.as<int32_t>(), m.d_col.as<int32_t>(), s->lapK.as<double>(), s->lapDinv.as<double>(),
                       s->lapFixed.as<uint8_t>(), s->lapR.as<D4>(), s->lapZ.as<D4>(), s->lapP.as<D4>(),
-                      s->lapAp.as<D4>(), s->lapPart.as<double>(), s->lapCg.p};
+                      s->lapAp.as<D4>(), s->lapPart.as<double>(), s->lapCg.p, s->force_lifting_timeout};
   LFX_TRY(lifting_solve(st, L, s->n_bnd, s->bnd_node.as<int32_t>(), s->bnd_val.as<D4>(), s->dnew.as<D4>(), 1e-12,
                         20000, &s->lifting_iters));
   const bool mixed = s->mixed();
@@ -2151,6 +2152,16 @@ lfx_status lfx_debug_cycle_timeout(lfx_state *s, int32_t on) {
     return LFX_ERR_INVALID_ARG;
   }
   s->pc64.force_cycle_timeout = s->pc32.force_cycle_timeout = s->pcbf.force_cycle_timeout = on != 0;
+  return LFX_OK;
+}
+
+lfx_status lfx_debug_lifting_timeout(lfx_state *s, int32_t on) {
+  clear_error();
+  if (!s) {
+    set_error("lfx_debug_lifting_timeout: NULL state");
+    return LFX_ERR_INVALID_ARG;
+  }
+  s->force_lifting_timeout = on != 0;
   return LFX_OK;
 }
 

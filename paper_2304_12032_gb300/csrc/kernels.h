@@ -176,6 +176,7 @@ struct LiftingView {
   D4 *r, *z, *p, *Ap;      // [V]
   double *part;            // lifting_part_entries(V)
   void *cg_state;          // lifting_cg_state_bytes()
+  bool force_timeout = false;   // tests: the grid-wide waits of the one-launch solve run out
 };
 lfx_status launch_lifting_matrix(cudaStream_t st, int64_t T, int64_t V, int64_t nnzb, const int32_t *slot,
                                  const int32_t *diag, const double *geo64, const float *geo_hi, const float *geo_lo,

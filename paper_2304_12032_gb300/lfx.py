@@ -134,6 +134,7 @@ _SIGS = {
     "lfx_debug_persistent_timeout": ([_P], ctypes.c_int32),
     "lfx_debug_staged_timeout": ([_P], ctypes.c_int32),
     "lfx_debug_cycle_timeout": ([_P, ctypes.c_int32], ctypes.c_int32),
+    "lfx_debug_lifting_timeout": ([_P, ctypes.c_int32], ctypes.c_int32),
     "lfx_debug_precond": ([_P, _DP, _DP, _DP, _DP], ctypes.c_int32),
     "lfx_debug_solve": ([_P, _DP, ctypes.POINTER(lfx_step_stats)], ctypes.c_int32),
     "lfx_set_allocator": ([ALLOC_FN, FREE_FN, _P], ctypes.c_int32),
@@ -553,6 +554,10 @@ class State:
     def debug_cycle_timeout(self, on):
         """Make the grid-wide waits of the persistent Krylov cycles run out from now on, or not any more."""
         _check(library().lfx_debug_cycle_timeout(self.h, int(on)))
+
+    def debug_lifting_timeout(self, on):
+        """Make the grid-wide waits of the moving mesh's lifting run out from now on, or not any more."""
+        _check(library().lfx_debug_lifting_timeout(self.h, int(on)))
 
     def debug_spmv(self, x):
         x = np.ascontiguousarray(x, dtype=np.float64).reshape(self.V, 4)

@@ -1,4 +1,4 @@
-"""The bounded waits of the persistent Krylov cycle, made to run out (a target that nothing reaches, a limit of
+"""The bounded waits of the persistent Krylov cycle and of the lifting, made to run out (a target that nothing reaches, a limit of
 milliseconds): the step reports LFX_ERR_TIMEOUT after a few launches instead of restarting an empty cycle until
 the host's own limit of 100,000, the state keeps its time level, and its next step equals a fresh state's."""
 import numpy as np
@@ -69,3 +69,31 @@ def test_cycle_waits_that_run_out_in_a_solve():
     st.debug_cycle_timeout(False)
     st.debug_assemble(apply_bcs=True)
     assert st.debug_solve()[1]["converged"]
+
+
+@pytest.mark.parametrize("n", [2, 9, 24])
+def test_lifting_waits_that_run_out(n):
+    """One CTA, fewer rows than CTAs, a full grid.  The repeated step extends linear boundary data to the linear
+    field, to the 1e-9 derived in the lifting's own test (two states' liftings differ in the last bits: their
+    matrices are summed in the order of atomic additions)."""
+    from paper_2304_12032_gb300 import lfx as L
+    from synthetic import cube_kuhn
+
+    m = cube_kuhn(n, seed=n)
+    prob = L.Problem(L.Mesh.from_synthetic(m), 1.0, 1.0, 1e-3, 1, [L.BC(tag=t, kind="nodal") for t in range(1, 7)], [],
+                     L.default_options(pin_pressure_node=0))
+    V = m.n_nodes
+    st = L.State(prob, np.zeros((1, V, 3)), np.zeros((1, V)), 0.0)
+    st.set_displacement(np.zeros((1, V, 3)))
+    d = m.nodes @ np.array([[0.02, 0.01, 0.0], [-0.01, 0.03, 0.0], [0.0, 0.02, -0.02]]) + 0.005
+    bd = np.unique(m.bfaces.ravel())
+    st.set_boundary_displacement(bd, d[bd])
+    st.debug_lifting_timeout(True)
+    for _ in range(2):
+        with pytest.raises(L.LfxError) as err:
+            st.step()
+        assert err.value.status == L.LFX_ERR_TIMEOUT and "gave up" in str(err.value)
+    assert not st.get_displacement()[0].any()              # the state keeps its time level
+    st.debug_lifting_timeout(False)
+    assert st.step(allow_not_converged=True)["t"] == 1e-3   # (and the prescribed data, for the repetition)
+    assert np.abs(st.get_displacement()[0] - d).max() <= 1e-9 * np.abs(d).max()
