@@ -2971,12 +2971,15 @@ bool ASimple<S, T>::cycle_ready() const {
 template <class S, class T>
 lfx_status ASimple<S, T>::cycle(cudaStream_t st, const int32_t *rowptr, const T *A, T *Vb, T *Zb, T *wk, T *x, KState *ks,
                                 KState *kseg, KState *parent, int m, int maxit) {
-  if (!cyc_sync.p) {
-    LFX_TRY(cyc_part.alloc(cycle_part_bytes(*plan)));
-    LFX_TRY(cyc_sync.alloc(sizeof(CycleSync)));
-    LFX_CUDA_TRY(cudaMemsetAsync(cyc_sync.p, 0, sizeof(CycleSync), st));
+  // (cyc_sync last: where it is, the others are; a step that failed at one of them is repeated from there)
+  if (!cyc_host) {
     LFX_CUDA_TRY(cudaMallocHost(&cyc_host, sizeof(CycleSync)));
     std::memset(cyc_host, 0, sizeof(CycleSync));
+  }
+  if (!cyc_part.p) LFX_TRY(cyc_part.alloc(cycle_part_bytes(*plan)));
+  if (!cyc_sync.p) {
+    LFX_TRY(cyc_sync.alloc(sizeof(CycleSync)));
+    LFX_CUDA_TRY(cudaMemsetAsync(cyc_sync.p, 0, sizeof(CycleSync), st));
   }
   CycleArgs<S, T> a{};
   a.V = V;
