@@ -646,8 +646,8 @@ __device__ __forceinline__ void dense_algebra(const CycleArgs<S, T> &A, unsigned
 }
 
 // The same for several segments in lockstep, a warp per segment, with the Hessenberg matrix and rotations in
-// the segments' status structs.  A segment that has converged keeps its count and solution; its rows go on
-// with basis vectors that nothing uses until every segment has.
+// the segments' status structs.  A segment that has converged keeps its count and solution; its rows meet the
+// others at their barriers with basis vectors of zeros until every segment has.
 template <class S, class T, int LPR>
 __device__ __forceinline__ void dense_algebra_seg(const CycleArgs<S, T> &A, unsigned rows_ctas) {
   using Sm = Sum<T>;
@@ -770,7 +770,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ T hs[kMaxRestart + 1];
   __shared__ SumT red[(kMaxRestart + 1) * kDots];
-  __shared__ int verdict, resident, solved;
+  __shared__ int verdict, resident, solved, over;   // over: this CTA's segment has converged (thread 0's)
   if (finished(A.ks)) return;
   const unsigned rows_ctas = gridDim.x - 1, cta = blockIdx.x;
   if (*(volatile const int *)&A.sync->error) {   // a wait of an earlier cycle gave up
@@ -850,6 +850,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
   }
   __syncthreads();
   if (tid == 0) {   // rows whose velocity records fit
+    over = 0;
     const int64_t most = A.f_bytes / (12 * sizeof(S));
     int lo = 0, hi = o.n;
     while (lo < hi) {
@@ -887,6 +888,8 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
       if (v == 0 && decide > 0) {
         if (!wait_for(&A.sync->progress, 2u * (unsigned)decide, A.polls)) v = 1;
         else if (ld_relaxed(&A.sync->progress) & 1u) v = 2;
+        // (not written again before this CTA has arrived at the end of the step)
+        if (v == 0 && A.n_seg > 1) over = *(volatile const int *)&A.kseg[A.cta_seg[cta]].done;
       }
       if (v == 1) atomicExch(&A.sync->error, 1);
       verdict = v;
@@ -1176,7 +1179,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
       for (int q = 16; q > 0; q >>= 1) Sm::join(a, Sm::shfl(a, q));
       if (lane == 0) {
         const T n2 = Sm::rounded(a);
-        hs[0] = n2 > T(0) ? T(1) / sqrt(n2) : T(0);
+        hs[0] = n2 > T(0) && !over ? T(1) / sqrt(n2) : T(0);
       }
     }
     __syncthreads();

@@ -41,3 +41,35 @@ def test_many_short_cycles_repeat_bit_for_bit():
         got.append(st.get())
     for u, p in got[1:]:
         assert np.array_equal(u, got[0][0]) and np.array_equal(p, got[0][1])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_hard_member_beside_easy_ones(precision):
+    """Members that converge early wait with zero basis vectors for the hardest one: each solution equals the
+    member's own solve (both to 1e-11 of the right-hand side; 1e-7 as in the batch test of the cycle), and the
+    batch takes no more steps than the hardest member alone, up to the different hierarchies."""
+    from paper_2304_12032_gb300 import lfx as L
+    from synthetic import batch, cube_kuhn
+
+    sizes, rng = (3, 16, 2, 4), np.random.default_rng(2)
+    ms = [cube_kuhn(n, seed=n) for n in sizes]
+    hist = [(rng.standard_normal((1, m.n_nodes, 3)), rng.standard_normal((1, m.n_nodes))) for m in ms]
+    opt = dict(precision=precision, gmres_rtol=1e-11, smoother_bf16=1)
+    bcs = [L.BC(tag=t, kind="noslip") for t in range(1, 6)] + [L.BC(tag=6, kind="neumann", time="constant", p=(0.0,))]
+
+    def solve(m, u, p):
+        prob = L.Problem(L.Mesh.from_synthetic(m), 1.0, 0.05, 1e-2, 1, bcs, [], L.default_options(**opt))
+        st = L.State(prob, u, p, 0.0)
+        return st.step(), *st.get()
+
+    union = batch(ms, tag_stride=0)
+    stats, u, p = solve(union, np.concatenate([h[0] for h in hist], axis=1), np.concatenate([h[1] for h in hist], axis=1))
+    assert stats["converged"]
+    off, steps = union.meta["node_offsets"], []
+    for i, m in enumerate(ms):
+        a, ui, pi = solve(m, *hist[i])
+        steps.append(a["iterations"])
+        sl = slice(off[i], off[i] + m.n_nodes)
+        assert rel(u[sl], ui) < 1e-7 and rel(p[sl], pi) < 1e-7
+    assert min(steps) < max(steps)
+    assert stats["iterations"] <= 1.25 * max(steps) + 4
