@@ -169,4 +169,22 @@ LFX_HD dd dd_rsqrt(dd x) {
   return y + y * (h * dd(0.5f, 0.0f));
 }
 
+// 1 / sqrt(hi + lo) rounded once to FP32, |lo| far below hi; 0 unless hi > 0 is finite.  An FP32 estimate y (relative
+// error up to 2^-22) and a Newton step y + y t / 2, t = 1 - (hi + lo) y^2 from the exact square of y: the step
+// leaves 3/8 t^2 < 2^-43.  hi is first brought near 1 by an even power of two where y^2 might leave the range.
+LFX_HD float inv_sqrt_once(float hi, float lo) {
+  if (!(hi > 0.0f && hi < HUGE_VALF)) return 0.0f;
+  const bool small = hi < 1e-24f, large = hi > 1e24f;
+  const float up = small ? 0x1p80f : (large ? 0x1p-80f : 1.0f), back = small ? 0x1p40f : (large ? 0x1p-40f : 1.0f);
+  hi = f_mul(hi, up);
+#ifdef __CUDA_ARCH__
+  const float y = rsqrtf(hi);
+#else
+  const float y = 1.0f / std::sqrt(hi);
+#endif
+  const dd q = two_prod(y, y);
+  const float t = f_fma(-f_mul(lo, up), q.hi, f_fma(-hi, q.lo, f_fma(-hi, q.hi, 1.0f)));
+  return f_mul(f_fma(f_mul(0.5f, y), t, y), back);
+}
+
 }  // namespace lfx
