@@ -882,14 +882,14 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
     if (tid == 0) o.sv[o.loc] = T(0);
     __syncthreads();
   };
-  unsigned target = 0;
+  unsigned target = A.unreachable;   // (0 but in tests)
   // grid barrier; with decide >= 0 also the verdict on that step: 0 go on, 1 a wait gave up, 2 the cycle has ended
   auto barrier = [&](int decide) -> int {
     __syncthreads();
     target += rows_ctas;
     if (tid == 0) {
       arrive(&A.sync->arrived);
-      int v = wait_for(&A.sync->arrived, target + A.unreachable, A.polls) ? 0 : 1;
+      int v = wait_for(&A.sync->arrived, target, A.polls) ? 0 : 1;
       if (v == 0 && decide > 0) {
         if (!wait_for(&A.sync->progress, 2u * (unsigned)decide, A.polls)) v = 1;
         else if (ld_relaxed(&A.sync->progress) & 1u) v = 2;
