@@ -146,7 +146,7 @@ struct lfx_problem {
   // assembly launch shape (LFX_ASM_*): options.assembly, or the autotuner's choice (0 until tuned),
   // with the tuning times (ms per assembly: colours, chunks, persistent) and the device copy of the
   // chunk colour offsets the persistent launch reads
-  std::mutex tune_mu;
+  mutable std::mutex tune_mu;
   int asm_mode = 0, asm_mode_newton = 0;   // launch shapes of the semi-implicit and Newton systems
   float asm_ms[3] = {0.0f, 0.0f, 0.0f}, asm_ms_newton[3] = {0.0f, 0.0f, 0.0f};
   DBuf d_chunk_color_off;
@@ -200,7 +200,8 @@ struct lfx_state {
   DBuf dhist[3], dnew, uale, xyz, xyz_hi, xyz_lo, geo64, geo_hi, geo_lo;
   DBuf lapK, lapDinv, lapFixed, lapR, lapZ, lapP, lapAp, lapPart, lapCg, bnd_node, bnd_val;
   // persistent assembly: grid-barrier counter and error word (device), the error word's host copy
-  DBuf asm_sync, gather;   // (gather: the gathered assembly's scratch)
+  DBuf asm_sync, gather;   // (gather: the gathered assembly's scratch, held while a launch shape in use needs it)
+  bool no_gather = false;  // it could not be had: the coloured form runs
   int *asm_err_host = nullptr;
   int asm_mode_used = 0;
   bool force_timeout = false;   // tests: make the persistent assembly's first grid-wide wait run out
@@ -1192,6 +1193,12 @@ lfx_status lfx_state_device_bytes(const lfx_state *s, int64_t *bytes) {
 static size_t gather_bytes(const Mesh &m) {
   return m.blk_run.empty() ? 0 : sizeof(double) * (16 * m.blk_run.size() + 4 * (size_t)m.pass_diag_off.back());
 }
+// whether a state of the problem takes that scratch: the persistent launch is a shape of its systems, or still
+// one of the shapes to be timed.  (tune_mu held)
+static bool gather_in_use(const lfx_problem *pb) {
+  auto may = [](int mode) { return mode == LFX_ASM_PERSISTENT || mode == LFX_ASM_AUTO; };
+  return may(pb->asm_mode) || (pb->opt.implicit && may(pb->asm_mode_newton));
+}
 
 // Assembly of the system for t^{n+1} = t + dt into vals64 / rhs, x0 = extrapolation.  With
 // newton, the Jacobian of the fully implicit formulation at the iterate held in xsol and the
@@ -1277,8 +1284,6 @@ static lfx_status assemble_system(lfx_state *s, bool apply_bcs, bool newton = fa
     CA.n_blocks = m.nnzb;
     CA.n_runs = (int64_t)m.blk_run.size();
     CA.n_diag = m.pass_diag_off.back();
-    if (!s->gather.p) LFX_TRY(s->gather.alloc(gather_bytes(m)));
-    CA.scratch = s->gather.p;
   }
   if (mixed) A.bad = pb->n_bad > 0 ? pb->d_bad.as<uint8_t>() : nullptr;   // badly shaped: FP64 geometry
   if (!s->asm_sync.p) {
@@ -1288,8 +1293,16 @@ static lfx_status assemble_system(lfx_state *s, bool apply_bcs, bool newton = fa
   }
   unsigned *barrier = s->asm_sync.as<unsigned>();
   int *err = reinterpret_cast<int *>(s->asm_sync.as<char>() + 32);
-  // one assembly of the semi-implicit system (or the Newton system) in launch shape `mode`
+  // one assembly of the semi-implicit system (or the Newton system) in launch shape `mode`; the persistent one
+  // gathers where its scratch can be had
   auto launch = [&](int mode) -> lfx_status {
+    if (mode == LFX_ASM_PERSISTENT && !m.blk_run.empty()) {
+      if (!s->gather.p && !s->no_gather && s->gather.alloc(gather_bytes(m)) != LFX_OK) {
+        s->no_gather = true;
+        clear_error();
+      }
+      CA.scratch = s->gather.p;
+    }
     if (mixed) {
       if (mode == LFX_ASM_COLORS)
         return launch_assemble<dd, float>(st, A, pb->P, m.color_off.data(), (int)m.color_off.size() - 1,
@@ -1336,6 +1349,7 @@ static lfx_status assemble_system(lfx_state *s, bool apply_bcs, bool newton = fa
         }
       }
       tuned = pick;
+      if (!gather_in_use(pb)) s->gather.release();   // (the candidate that used it has ended)
     }
     mode = tuned;
   }
@@ -1430,7 +1444,10 @@ int64_t lfx_internal_state_bytes_estimate(const lfx_problem *pb, int64_t *V_out,
   if (sigma_out) *sigma_out = sigma;
   const int64_t v64 = 32 * V, v32 = 16 * V;
   int64_t b = (sigma + 3) * v64 + 64 * (int64_t)pb->dir_node.size() + 8 * m.n_comp;
-  b += (int64_t)gather_bytes(m);                             // gathered assembly
+  {
+    std::lock_guard<std::mutex> lk(pb->tune_mu);
+    if (gather_in_use(pb)) b += (int64_t)gather_bytes(m);    // gathered assembly
+  }
   b += 9 * 152 * 8 * 65;                                     // partial sums of the persistent Krylov cycle
   b += sigma * v64;                                          // caller-layout staging (history in, solution out)
   b += 128 * nnzb;                                           // FP64 or double-float matrix
