@@ -510,6 +510,14 @@ static std::complex<double> bessel_j1(std::complex<double> z) {
   return sum;
 }
 
+// whether the problem's Krylov solves may run as persistent cycles (what ASimple::plan_cycles and Gmres::run_cycle
+// ask for): without it no row partition is made
+static bool cycles_wanted(const lfx_problem *pb) {
+  const lfx_options &o = pb->opt;
+  const bool cgs2 = o.precision == LFX_PREC_MIXED ? o.reorthogonalize == 2 : o.reorthogonalize != 0;
+  return o.s_smoother == LFX_SMOOTH_AMG && o.s_steps == 1 && o.f_steps >= 2 && !cgs2 && pb->n_r1_tags == 0;
+}
+
 lfx_status lfx_problem_create(const lfx_mesh *mesh, double rho, double mu, double dt, int32_t bdf_order,
                               const lfx_bc *bcs, int32_t n_bcs, const lfx_riis *riis, int32_t n_riis,
                               const lfx_options *opt, lfx_problem **out) {
@@ -958,13 +966,17 @@ lfx_status lfx_problem_create(const lfx_mesh *mesh, double rho, double mu, doubl
   LFX_CUDA_TRY(cudaMemcpy(pb->d_chunk_color_off.p, m.chunk_color_off.data(), sizeof(int32_t) * m.chunk_color_off.size(),
                           cudaMemcpyHostToDevice));
   pb->asm_mode = pb->asm_mode_newton = o.assembly;
-  // the row partition of the persistent Krylov cycle
-  if (o.s_smoother == LFX_SMOOTH_AMG) {
+  // the row partition of the persistent Krylov cycle (where there is no memory for it the solves run step by step)
+  if (cycles_wanted(pb.get())) {
     int ctas = 0;
     const CycleMap *map = nullptr;
     if (o.precision == LFX_PREC_MIXED) LFX_TRY(cycle_ctas<float>(V, &ctas));
     else LFX_TRY(cycle_ctas<double>(V, &ctas));
-    if (ctas > 0) LFX_TRY(mesh_cycle_map(m, ctas, m.n_comp > 1 && o.batch_segmented, &map));
+    if (ctas > 0) {
+      const lfx_status rc = mesh_cycle_map(m, ctas, m.n_comp > 1 && o.batch_segmented, &map);
+      if (rc == LFX_ERR_OOM) clear_error();
+      else LFX_TRY(rc);
+    }
   }
   *out = pb.release();
   return LFX_OK;
@@ -1505,7 +1517,7 @@ static lfx_status setup_asimple(lfx_state *s, ASimple<S, T> &pc) {
   lfx_problem *pb = s->pb;
   const lfx_options &o = pb->opt;
   const Mesh &m = pb->mesh->m;
-  pc.plan_cycles(m, m.n_comp > 1 && o.batch_segmented);
+  if (cycles_wanted(pb)) pc.plan_cycles(m, m.n_comp > 1 && o.batch_segmented);
   if (s->mixed())
     LFX_TRY(pc.setup_split(s->stream, s->view<float>(s->vals32), m.nnzb));   // from the high parts
   else

@@ -4,10 +4,12 @@
 // transpose map, outward boundary faces, and a greedy element colouring so that elements of one
 // colour share no node and their block updates need no atomics.
 #include <algorithm>
-#include <thread>
+#include <atomic>
 #include <cmath>
 #include <cstring>
+#include <new>
 #include <numeric>
+#include <thread>
 
 #include "lfx_internal.h"
 
@@ -678,37 +680,42 @@ static void cycle_ranges(const Mesh &m, int ctas, bool segments, std::vector<int
   }
 }
 
+// the halo of every CTA and the local column indices, CTAs dealt to host threads (as many as can be had)
 static void cycle_map_lists(const Mesh &m, const std::vector<int32_t> &row_off, std::vector<int32_t> &halo_off,
                             std::vector<int32_t> &halo, std::vector<uint16_t> &lcol, int *max_rows, int *max_loc) {
   const int ctas = (int)row_off.size() - 1;
   std::vector<std::vector<int32_t>> lists(ctas);
   lcol.assign((size_t)std::max<int64_t>(m.nnzb, 1), 0);
-  const int nt = (int)std::min<unsigned>(std::max(1u, std::thread::hardware_concurrency()), 16u);
-  auto work = [&](int t) {
-    std::vector<int32_t> local((size_t)m.V, -1);
-    for (int b = t; b < ctas; b += nt) {
-      const int32_t r0 = row_off[b], r1 = row_off[b + 1];
-      std::vector<int32_t> &h = lists[b];
-      for (int32_t k = m.row_ptr[r0]; k < m.row_ptr[r1]; ++k) {
-        const int32_t c = m.col_idx[k];
-        if ((c < r0 || c >= r1) && local[c] < 0) {
-          local[c] = 0;
-          h.push_back(c);
+  std::atomic<int> next{0};
+  std::atomic<bool> failed{false};
+  auto work = [&]() noexcept {
+    try {
+      for (int b = next++; b < ctas; b = next++) {
+        const int32_t r0 = row_off[b], r1 = row_off[b + 1];
+        std::vector<int32_t> &h = lists[b];
+        for (int32_t k = m.row_ptr[r0]; k < m.row_ptr[r1]; ++k)
+          if (m.col_idx[k] < r0 || m.col_idx[k] >= r1) h.push_back(m.col_idx[k]);
+        std::sort(h.begin(), h.end());
+        h.erase(std::unique(h.begin(), h.end()), h.end());
+        for (int32_t k = m.row_ptr[r0]; k < m.row_ptr[r1]; ++k) {
+          const int32_t c = m.col_idx[k];
+          const int64_t l = c >= r0 && c < r1 ? c - r0 : (r1 - r0) + (std::lower_bound(h.begin(), h.end(), c) - h.begin());
+          lcol[k] = (uint16_t)l;   // (unused when max_loc exceeds 16 bits)
         }
       }
-      std::sort(h.begin(), h.end());
-      for (size_t i = 0; i < h.size(); ++i) local[h[i]] = (int32_t)(r1 - r0 + (int64_t)i);
-      for (int32_t k = m.row_ptr[r0]; k < m.row_ptr[r1]; ++k) {
-        const int32_t c = m.col_idx[k];
-        lcol[k] = (uint16_t)(c >= r0 && c < r1 ? c - r0 : local[c]);   // (unused when max_loc exceeds 16 bits)
-      }
-      for (const int32_t c : h) local[c] = -1;
+    } catch (const std::bad_alloc &) {
+      failed = true;
     }
   };
   std::vector<std::thread> th;
-  for (int t = 1; t < nt; ++t) th.emplace_back(work, t);
-  work(0);
+  try {
+    const int nt = (int)std::min<unsigned>(std::max(1u, std::thread::hardware_concurrency()), 16u);
+    for (int t = 1; t < nt; ++t) th.emplace_back(work);
+  } catch (const std::exception &) {   // no more threads: those that run and this one do the work
+  }
+  work();
   for (auto &t : th) t.join();
+  if (failed) throw std::bad_alloc();
   halo_off.assign(1, 0);
   halo.clear();
   *max_rows = *max_loc = 0;
@@ -735,8 +742,14 @@ lfx_status mesh_cycle_map(const Mesh &m, int ctas, bool segments, const CycleMap
   if (!c) return LFX_ERR_OOM;
   std::vector<int32_t> row_off, cta_seg, seg_off, off, halo;
   std::vector<uint16_t> lcol;
-  cycle_ranges(m, ctas, segments, row_off, cta_seg, seg_off);
-  cycle_map_lists(m, row_off, off, halo, lcol, &c->max_rows, &c->max_loc);
+  try {
+    cycle_ranges(m, ctas, segments, row_off, cta_seg, seg_off);
+    cycle_map_lists(m, row_off, off, halo, lcol, &c->max_rows, &c->max_loc);
+    m.cycle_maps.reserve(m.cycle_maps.size() + 1);
+  } catch (const std::bad_alloc &) {
+    set_error("row partition of the Krylov cycle: out of host memory");
+    return LFX_ERR_OOM;
+  }
   auto up = [](DBuf &d, const void *src, size_t bytes) -> lfx_status {
     LFX_TRY(d.alloc(std::max<size_t>(bytes, 16)));
     if (bytes) LFX_CUDA_TRY(cudaMemcpy(d.p, src, bytes, cudaMemcpyHostToDevice));
