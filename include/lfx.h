@@ -108,6 +108,22 @@ lfx_status lfx_mesh_get_chunks(const lfx_mesh *mesh, int64_t sizes[5], int32_t *
  * maximum blocks per tile}.  Non-NULL arrays receive tile_row [tiles+1] (the internal block-row
  * range of each tile) and row_node [n_nodes] (the caller node of each internal block row). */
 lfx_status lfx_mesh_get_row_tiles(const lfx_mesh *mesh, int64_t sizes[3], int32_t *tile_row, int32_t *row_node);
+/* The row partition of the persistent Krylov cycle for `ctas` CTAs, for inspection and tests (host, no
+ * device work); with segments = 1 every CTA's rows lie in one connected piece (at least as many CTAs as
+ * pieces).  sizes = {segments, most rows of a CTA, most rows and halo rows together, halo rows of all
+ * CTAs}.  Non-NULL arrays receive row_off [ctas+1] (internal block rows), cta_seg [ctas], halo_off [ctas+1]
+ * and halo (rows of other CTAs that a CTA's blocks read, ascending), and local_col [nnz_blocks] (each
+ * block's column, in internal block order, as an index into its CTA's own rows followed by its halo;
+ * the low 16 bits where the third size exceeds 65535, and no cycle runs). */
+lfx_status lfx_mesh_get_cycle_partition(const lfx_mesh *mesh, int32_t ctas, int32_t segments, int64_t sizes[4],
+                                        int32_t *row_off, int32_t *cta_seg, int32_t *halo_off, int32_t *halo,
+                                        uint16_t *local_col);
+/* The tables of the gathered assembly, for inspection and tests (host, no device work).  sizes = {runs (0:
+ * the mesh is assembled colour by colour), diagonal runs}.  Non-NULL arrays receive run_block [runs] (the
+ * internal block of each run of lfx_mesh_get_chunks), block_off [nnz_blocks+1] and block_run [runs] (the runs
+ * of each block, ascending), run_diag [runs] (number of a diagonal run, else -1). */
+lfx_status lfx_mesh_get_gather(const lfx_mesh *mesh, int64_t sizes[2], int32_t *run_block, int32_t *block_off,
+                               int32_t *block_run, int32_t *run_diag);
 
 /* ------------------------------------------------------------------------------------------
  * Problem: physics (Section 2.1), boundary conditions (Section 2.2), RIIS surfaces (Eq. riis),
@@ -398,6 +414,10 @@ lfx_status lfx_debug_persistent_timeout(lfx_state *state);
  * returns.  LFX_ERR_TIMEOUT is the expected result; the state stays usable (the next lfx_step
  * assembles anew).  Needs a mixed-precision state with smoother_bf16 and staged_f set. */
 lfx_status lfx_debug_staged_timeout(lfx_state *state);
+/* The shape of the state's persistent Krylov cycle after a step or solve: plan = {CTAs with rows (0: the
+ * solves run step by step), lanes per row, row data left in global memory (0 none, 1 some, 2 all), segments,
+ * most rows of a CTA, most rows and halo rows together}.  Host-only. */
+lfx_status lfx_debug_cycle_plan(const lfx_state *state, int32_t plan[6]);
 /* on = 1: from now on the grid-wide waits of the state's persistent Krylov cycles get a target that
  * nothing reaches and a limit of milliseconds, so that they run out (LFX_ERR_TIMEOUT from lfx_step);
  * on = 0: back to normal.  Host-only. */

@@ -377,6 +377,52 @@ lfx_status lfx_mesh_get_row_tiles(const lfx_mesh *mesh, int64_t sizes[3], int32_
   return LFX_OK;
 }
 
+lfx_status lfx_mesh_get_cycle_partition(const lfx_mesh *mesh, int32_t ctas, int32_t segments, int64_t sizes[4],
+                                        int32_t *row_off, int32_t *cta_seg, int32_t *halo_off, int32_t *halo,
+                                        uint16_t *local_col) {
+  clear_error();
+  if (!mesh || !sizes || ctas < 1 || (segments && mesh->m.n_comp > ctas)) {
+    set_error("lfx_mesh_get_cycle_partition: NULL argument, no CTAs, or more pieces than CTAs");
+    return LFX_ERR_INVALID_ARG;
+  }
+  CycleLists L;
+  LFX_TRY(cycle_lists(mesh->m, ctas, segments != 0, L));
+  sizes[0] = (int64_t)L.seg_off.size() - 1;
+  sizes[1] = L.max_rows;
+  sizes[2] = L.max_loc;
+  sizes[3] = (int64_t)L.halo.size();
+  auto put = [](auto *dst, const auto &v, size_t n) {
+    if (dst) std::copy(v.begin(), v.begin() + (ptrdiff_t)n, dst);
+  };
+  put(row_off, L.row_off, L.row_off.size());
+  put(cta_seg, L.cta_seg, L.cta_seg.size());
+  put(halo_off, L.halo_off, L.halo_off.size());
+  put(halo, L.halo, L.halo.size());
+  put(local_col, L.lcol, (size_t)mesh->m.nnzb);
+  return LFX_OK;
+}
+
+lfx_status lfx_mesh_get_gather(const lfx_mesh *mesh, int64_t sizes[2], int32_t *run_block, int32_t *block_off,
+                               int32_t *block_run, int32_t *run_diag) {
+  clear_error();
+  if (!mesh || !sizes) {
+    set_error("lfx_mesh_get_gather: NULL argument");
+    return LFX_ERR_INVALID_ARG;
+  }
+  const Mesh &m = mesh->m;
+  sizes[0] = (int64_t)m.blk_run.size();
+  sizes[1] = m.blk_run.empty() ? 0 : m.pass_diag_off.back();
+  if (m.blk_run.empty()) return LFX_OK;
+  auto put = [](int32_t *dst, const std::vector<int32_t> &v) {
+    if (dst) std::copy(v.begin(), v.end(), dst);
+  };
+  put(run_block, m.run_block);
+  put(block_off, m.blk_off);
+  put(block_run, m.blk_run);
+  put(run_diag, m.run_diag);
+  return LFX_OK;
+}
+
 lfx_status lfx_mesh_get_chunks(const lfx_mesh *mesh, int64_t sizes[5], int32_t *elem_old, int32_t *chunk_elem_off,
                                int32_t *chunk_color_off, int32_t *chunk_pass_off, uint16_t *pass_code,
                                int32_t *pass_run_off, uint16_t *run_meta, int32_t *run_row, int32_t *run_col) {
@@ -2171,6 +2217,29 @@ lfx_status lfx_debug_staged_timeout(lfx_state *s) {
     set_error("staged velocity smoothing pass: a wait for a tile gave up");
     return LFX_ERR_TIMEOUT;
   }
+  return LFX_OK;
+}
+
+lfx_status lfx_debug_cycle_plan(const lfx_state *s, int32_t plan[6]) {
+  clear_error();
+  if (!s || !plan) {
+    set_error("lfx_debug_cycle_plan: NULL argument");
+    return LFX_ERR_INVALID_ARG;
+  }
+  std::fill(plan, plan + 6, 0);
+  auto put = [plan](const auto &pc) {
+    if (!pc.plan || !pc.cycle_ready()) return;
+    const CyclePlan &p = *pc.plan;
+    plan[0] = p.rows_ctas;
+    plan[1] = p.lanes;
+    plan[2] = p.spill;
+    plan[3] = p.map->n_seg;
+    plan[4] = p.map->max_rows;
+    plan[5] = p.map->max_loc;
+  };
+  put(s->pc64);
+  put(s->pc32);
+  put(s->pcbf);
   return LFX_OK;
 }
 

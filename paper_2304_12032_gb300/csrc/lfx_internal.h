@@ -100,6 +100,12 @@ struct DBuf {
 // The block rows dealt to `ctas` CTAs (consecutive ranges of nearly equal size; with segments each CTA owns
 // rows of one connected piece only), each with the list of the rows of other CTAs that its blocks read (its
 // halo, ascending), and every block's column as an index into own rows followed by the halo.
+// (CycleLists on the host, CycleMap on the device.)
+struct CycleLists {
+  std::vector<int32_t> row_off, cta_seg, seg_off, halo_off, halo;
+  std::vector<uint16_t> lcol;
+  int max_rows = 0, max_loc = 0;
+};
 struct CycleMap {
   int ctas = 0, n_seg = 1, max_rows = 0, max_loc = 0;   // max_loc: largest rows + halo (16-bit local indices)
   DBuf row_off, cta_seg, seg_off;            // int32 [ctas + 1], [ctas], [n_seg + 1] (CTAs of a segment)
@@ -180,6 +186,8 @@ struct Mesh {
 lfx_status build_mesh(const double *nodes, int64_t n_nodes, const int32_t *tets, int64_t n_tets,
                       const int32_t *bfaces, const int32_t *tags, int64_t n_bfaces, Mesh &m);
 lfx_status upload_mesh(Mesh &m);
+// the lists of a CTA count (host only; not more segments than CTAs)
+lfx_status cycle_lists(const Mesh &m, int ctas, bool segments, CycleLists &L);
 // the mesh's map for a CTA count, with or without segments (host lists, uploaded); it lives as long as the mesh.
 // *out is null when there are more pieces than CTAs.
 lfx_status mesh_cycle_map(const Mesh &m, int ctas, bool segments, const CycleMap **out);

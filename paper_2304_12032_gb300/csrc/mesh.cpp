@@ -655,8 +655,7 @@ lfx_status upload_mesh(Mesh &m) {
 
 // row ranges of the CTAs, and the CTA ranges of the segments: one more CTA at a time to the piece with the
 // most rows per CTA
-static void cycle_ranges(const Mesh &m, int ctas, bool segments, std::vector<int32_t> &row_off,
-                         std::vector<int32_t> &cta_seg, std::vector<int32_t> &seg_off) {
+static void cycle_ranges(const Mesh &m, int ctas, bool segments, CycleLists &L) {
   const std::vector<int32_t> all{0, (int32_t)m.V};
   const std::vector<int32_t> &off = segments ? m.comp_off : all;
   const int ns = (int)off.size() - 1;
@@ -667,25 +666,25 @@ static void cycle_ranges(const Mesh &m, int ctas, bool segments, std::vector<int
       if ((int64_t)(off[c + 1] - off[c]) * n[best] > (int64_t)(off[best + 1] - off[best]) * n[c]) best = c;
     ++n[best];
   }
-  row_off.assign(1, 0);
-  cta_seg.clear();
-  seg_off.assign(1, 0);
+  L.row_off.assign(1, 0);
+  L.cta_seg.clear();
+  L.seg_off.assign(1, 0);
   for (int c = 0; c < ns; ++c) {
     const int64_t rows = off[c + 1] - off[c];
     for (int b = 0; b < n[c]; ++b) {
-      row_off.push_back(off[c] + (int32_t)(rows * (b + 1) / n[c]));
-      cta_seg.push_back(c);
+      L.row_off.push_back(off[c] + (int32_t)(rows * (b + 1) / n[c]));
+      L.cta_seg.push_back(c);
     }
-    seg_off.push_back((int32_t)cta_seg.size());
+    L.seg_off.push_back((int32_t)L.cta_seg.size());
   }
 }
 
 // the halo of every CTA and the local column indices, CTAs dealt to host threads (as many as can be had)
-static void cycle_map_lists(const Mesh &m, const std::vector<int32_t> &row_off, std::vector<int32_t> &halo_off,
-                            std::vector<int32_t> &halo, std::vector<uint16_t> &lcol, int *max_rows, int *max_loc) {
+static void cycle_halos(const Mesh &m, CycleLists &L) {
+  const std::vector<int32_t> &row_off = L.row_off;
   const int ctas = (int)row_off.size() - 1;
   std::vector<std::vector<int32_t>> lists(ctas);
-  lcol.assign((size_t)std::max<int64_t>(m.nnzb, 1), 0);
+  L.lcol.assign((size_t)std::max<int64_t>(m.nnzb, 1), 0);
   std::atomic<int> next{0};
   std::atomic<bool> failed{false};
   auto work = [&]() noexcept {
@@ -700,7 +699,7 @@ static void cycle_map_lists(const Mesh &m, const std::vector<int32_t> &row_off, 
         for (int32_t k = m.row_ptr[r0]; k < m.row_ptr[r1]; ++k) {
           const int32_t c = m.col_idx[k];
           const int64_t l = c >= r0 && c < r1 ? c - r0 : (r1 - r0) + (std::lower_bound(h.begin(), h.end(), c) - h.begin());
-          lcol[k] = (uint16_t)l;   // (unused when max_loc exceeds 16 bits)
+          L.lcol[k] = (uint16_t)l;   // (unused when max_loc exceeds 16 bits)
         }
       }
     } catch (const std::bad_alloc &) {
@@ -716,16 +715,27 @@ static void cycle_map_lists(const Mesh &m, const std::vector<int32_t> &row_off, 
   work();
   for (auto &t : th) t.join();
   if (failed) throw std::bad_alloc();
-  halo_off.assign(1, 0);
-  halo.clear();
-  *max_rows = *max_loc = 0;
+  L.halo_off.assign(1, 0);
+  L.halo.clear();
+  L.max_rows = L.max_loc = 0;
   for (int b = 0; b < ctas; ++b) {
     const int rows = row_off[b + 1] - row_off[b];
-    halo.insert(halo.end(), lists[b].begin(), lists[b].end());
-    halo_off.push_back((int32_t)halo.size());
-    *max_rows = std::max(*max_rows, rows);
-    *max_loc = std::max(*max_loc, rows + (int)lists[b].size());
+    L.halo.insert(L.halo.end(), lists[b].begin(), lists[b].end());
+    L.halo_off.push_back((int32_t)L.halo.size());
+    L.max_rows = std::max(L.max_rows, rows);
+    L.max_loc = std::max(L.max_loc, rows + (int)lists[b].size());
   }
+}
+
+lfx_status cycle_lists(const Mesh &m, int ctas, bool segments, CycleLists &L) {
+  try {
+    cycle_ranges(m, ctas, segments, L);
+    cycle_halos(m, L);
+  } catch (const std::bad_alloc &) {
+    set_error("row partition of the Krylov cycle: out of host memory");
+    return LFX_ERR_OOM;
+  }
+  return LFX_OK;
 }
 
 lfx_status mesh_cycle_map(const Mesh &m, int ctas, bool segments, const CycleMap **out) {
@@ -740,27 +750,21 @@ lfx_status mesh_cycle_map(const Mesh &m, int ctas, bool segments, const CycleMap
     }
   std::unique_ptr<CycleMap> c(new (std::nothrow) CycleMap);
   if (!c) return LFX_ERR_OOM;
-  std::vector<int32_t> row_off, cta_seg, seg_off, off, halo;
-  std::vector<uint16_t> lcol;
-  try {
-    cycle_ranges(m, ctas, segments, row_off, cta_seg, seg_off);
-    cycle_map_lists(m, row_off, off, halo, lcol, &c->max_rows, &c->max_loc);
-    m.cycle_maps.reserve(m.cycle_maps.size() + 1);
-  } catch (const std::bad_alloc &) {
-    set_error("row partition of the Krylov cycle: out of host memory");
-    return LFX_ERR_OOM;
-  }
+  CycleLists L;
+  LFX_TRY(cycle_lists(m, ctas, segments, L));
+  c->max_rows = L.max_rows;
+  c->max_loc = L.max_loc;
   auto up = [](DBuf &d, const void *src, size_t bytes) -> lfx_status {
     LFX_TRY(d.alloc(std::max<size_t>(bytes, 16)));
     if (bytes) LFX_CUDA_TRY(cudaMemcpy(d.p, src, bytes, cudaMemcpyHostToDevice));
     return LFX_OK;
   };
-  LFX_TRY(up(c->row_off, row_off.data(), sizeof(int32_t) * row_off.size()));
-  LFX_TRY(up(c->cta_seg, cta_seg.data(), sizeof(int32_t) * cta_seg.size()));
-  LFX_TRY(up(c->seg_off, seg_off.data(), sizeof(int32_t) * seg_off.size()));
-  LFX_TRY(up(c->halo_off, off.data(), sizeof(int32_t) * off.size()));
-  LFX_TRY(up(c->halo, halo.data(), sizeof(int32_t) * halo.size()));
-  LFX_TRY(up(c->lcol, lcol.data(), sizeof(uint16_t) * lcol.size()));
+  LFX_TRY(up(c->row_off, L.row_off.data(), sizeof(int32_t) * L.row_off.size()));
+  LFX_TRY(up(c->cta_seg, L.cta_seg.data(), sizeof(int32_t) * L.cta_seg.size()));
+  LFX_TRY(up(c->seg_off, L.seg_off.data(), sizeof(int32_t) * L.seg_off.size()));
+  LFX_TRY(up(c->halo_off, L.halo_off.data(), sizeof(int32_t) * L.halo_off.size()));
+  LFX_TRY(up(c->halo, L.halo.data(), sizeof(int32_t) * L.halo.size()));
+  LFX_TRY(up(c->lcol, L.lcol.data(), sizeof(uint16_t) * L.lcol.size()));
   c->ctas = ctas;
   c->n_seg = n_seg;
   *out = c.get();

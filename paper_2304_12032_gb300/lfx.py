@@ -110,6 +110,9 @@ _SIGS = {
     "lfx_mesh_get_chunks": ([_P, _LP, _IP, _IP, _IP, _IP, ctypes.POINTER(ctypes.c_uint16), _IP,
                              ctypes.POINTER(ctypes.c_uint16), _IP, _IP], ctypes.c_int32),
     "lfx_mesh_get_row_tiles": ([_P, _LP, _IP, _IP], ctypes.c_int32),
+    "lfx_mesh_get_cycle_partition": ([_P, ctypes.c_int32, ctypes.c_int32, _LP, _IP, _IP, _IP, _IP,
+                                      ctypes.POINTER(ctypes.c_uint16)], ctypes.c_int32),
+    "lfx_mesh_get_gather": ([_P, _LP, _IP, _IP, _IP, _IP], ctypes.c_int32),
     "lfx_options_default": ([ctypes.POINTER(lfx_options)], None),
     "lfx_problem_create": ([_P, ctypes.c_double, ctypes.c_double, ctypes.c_double, ctypes.c_int32,
                             ctypes.POINTER(lfx_bc), ctypes.c_int32, ctypes.POINTER(lfx_riis), ctypes.c_int32,
@@ -133,6 +136,7 @@ _SIGS = {
     "lfx_debug_assemble_newton": ([_P, _DP, _DP, _DP], ctypes.c_int32),
     "lfx_debug_persistent_timeout": ([_P], ctypes.c_int32),
     "lfx_debug_staged_timeout": ([_P], ctypes.c_int32),
+    "lfx_debug_cycle_plan": ([_P, _IP], ctypes.c_int32),
     "lfx_debug_cycle_timeout": ([_P, ctypes.c_int32], ctypes.c_int32),
     "lfx_debug_lifting_timeout": ([_P, ctypes.c_int32], ctypes.c_int32),
     "lfx_debug_precond": ([_P, _DP, _DP, _DP, _DP], ctypes.c_int32),
@@ -336,6 +340,33 @@ class Mesh:
         _check(lib.lfx_mesh_get_row_tiles(self.h, sz.ctypes.data_as(_LP), _i(tile_row) if n else None, _i(row_node)))
         return {"tile_row": tile_row if n else np.zeros(0, np.int32), "row_node": row_node,
                 "max_rows": int(sz[1]), "max_blocks": int(sz[2])}
+
+    def cycle_partition(self, ctas, segments=False) -> dict:
+        """The persistent Krylov cycle's row partition (see lfx_mesh_get_cycle_partition)."""
+        get = library().lfx_mesh_get_cycle_partition
+        sz = np.zeros(4, dtype=np.int64)
+        _check(get(self.h, ctas, int(segments), sz.ctypes.data_as(_LP), None, None, None, None, None))
+        out = {"row_off": np.zeros(ctas + 1, np.int32), "cta_seg": np.zeros(ctas, np.int32),
+               "halo_off": np.zeros(ctas + 1, np.int32), "halo": np.zeros(max(int(sz[3]), 1), np.int32),
+               "local_col": np.zeros(self.info()["nnz_blocks"], np.uint16)}
+        _check(get(self.h, ctas, int(segments), sz.ctypes.data_as(_LP), _i(out["row_off"]), _i(out["cta_seg"]),
+                   _i(out["halo_off"]), _i(out["halo"]),
+                   out["local_col"].ctypes.data_as(ctypes.POINTER(ctypes.c_uint16))))
+        out["halo"] = out["halo"][:int(sz[3])]
+        return dict(out, segments=int(sz[0]), max_rows=int(sz[1]), max_loc=int(sz[2]))
+
+    def gather(self) -> dict:
+        """The gathered assembly's tables (see lfx_mesh_get_gather); empty where the mesh has none."""
+        get = library().lfx_mesh_get_gather
+        sz = np.zeros(2, dtype=np.int64)
+        _check(get(self.h, sz.ctypes.data_as(_LP), None, None, None, None))
+        n = int(sz[0])
+        if n == 0:
+            return {}
+        out = {"run_block": np.zeros(n, np.int32), "block_off": np.zeros(self.info()["nnz_blocks"] + 1, np.int32),
+               "block_run": np.zeros(n, np.int32), "run_diag": np.zeros(n, np.int32)}
+        _check(get(self.h, sz.ctypes.data_as(_LP), *(_i(out[k]) for k in ("run_block", "block_off", "block_run", "run_diag"))))
+        return dict(out, diagonal_runs=int(sz[1]))
 
     def chunks(self) -> dict:
         """The chunked assembly's tables (see lfx_mesh_get_chunks)."""
@@ -550,6 +581,12 @@ class State:
     def debug_staged_timeout(self):
         """Status of one BF16 preconditioner application whose staged-tile waits are made to run out."""
         return library().lfx_debug_staged_timeout(self.h)
+
+    def debug_cycle_plan(self) -> dict:
+        """Shape of the persistent Krylov cycle after a step (see lfx_debug_cycle_plan); ctas 0: step by step."""
+        p = np.zeros(6, np.int32)
+        _check(library().lfx_debug_cycle_plan(self.h, _i(p)))
+        return dict(zip(("ctas", "lanes", "spill", "segments", "max_rows", "max_loc"), p.tolist()))
 
     def debug_cycle_timeout(self, on):
         """Make the grid-wide waits of the persistent Krylov cycles run out from now on, or not any more."""

@@ -64,3 +64,34 @@ def test_a_partition_that_cannot_be_had_leaves_the_step_by_step_form(opts):
     assert hook.refused >= 1 and launches > 10 * its
     for a, b in zip(got, want):
         assert np.linalg.norm(a - b) <= 1e-6 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("n,precision,lanes,spill", [
+    (2, "fp64", 16, 0), (15, "fp64", 16, 0), (16, "fp64", 4, 0), (20, "mixed", 16, 0), (21, "mixed", 8, 0),
+    (26, "mixed", 4, 0), (56, "fp64", 4, 1), (70, "mixed", 4, 1), (84, "mixed", 4, 2)])
+def test_shapes_of_the_cycle_tests(n, precision, lanes, spill):
+    """The sizes at which the cycle is compared with the launches run the shapes that they are meant for."""
+    case = C.beltrami_case(n, seed=n)
+    mesh, _, st = C.gpu_state(case, precision=precision, smoother_bf16=1, assembly="chunks", gmres_rtol=1e-6)
+    assert st.debug_cycle_plan()["ctas"] == 0          # (not planned before the first set-up)
+    st.step()
+    p = st.debug_cycle_plan()
+    V = case.mesh.n_nodes
+    assert p["ctas"] == max(1, min(151, V // (8 if precision == "fp64" else 32)))
+    assert (p["lanes"], p["spill"], p["segments"]) == (lanes, spill, 1)
+    part = mesh.cycle_partition(p["ctas"])
+    assert (part["max_rows"], part["max_loc"]) == (p["max_rows"], p["max_loc"])
+
+
+@pytest.mark.parametrize("opts", [{}, MIXED], ids=["fp64", "mixed"])
+def test_shape_of_a_batch(opts):
+    from paper_2304_12032_gb300 import lfx as L
+    from synthetic import batch, cube_kuhn
+
+    m = batch([cube_kuhn(n, seed=n) for n in (2, 3, 9, 14)], tag_stride=0)
+    bcs = [L.BC(tag=t, kind="noslip") for t in range(1, 6)] + [L.BC(tag=6, kind="neumann", time="constant", p=(0.0,))]
+    for segmented in (1, 0):
+        prob = L.Problem(L.Mesh.from_synthetic(m), 1.0, 0.05, 1e-2, 1, bcs, [], L.default_options(batch_segmented=segmented, **opts))
+        st = L.State(prob, np.ones((1, m.n_nodes, 3)), np.zeros((1, m.n_nodes)), 0.0)
+        st.step()
+        assert st.debug_cycle_plan()["segments"] == (4 if segmented else 1)
