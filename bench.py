@@ -211,7 +211,11 @@ def kernel_rooflines(stats, T, V, nnzb, prec, bf16=True):
     staged = dd and bf16
     # the persistent Krylov cycle times all its passes by its own clock; step by step, one application's
     cycle = any(s["n_fpass"] > F_STEPS - 2 for s in stats)
-    clock = "the kernel's own clock around the pass (grid-wide wait included), mean over all of them"
+    clock = "the kernel's own clock from one grid-wide wait to the end of the next, mean over all of them"
+    clock_product = ("the kernel's own clock, the slowest CTA's product (copy of its halo included, the grid-wide wait "
+                     "after it not), mean over all of them")
+    reuse = ("algorithmic bytes at the pass's rate, not DRAM traffic: part of the records stays in shared memory and "
+             "the rest largely in L2, so the fraction is not a share of the HBM rate")
     f_bytes = nnzb * (12 * sf + (0 if staged else 4)) + 4 * (V + 1) + V * 4 * sx * 7
     fpass = None
     if f_ms > 0:
@@ -228,6 +232,8 @@ def kernel_rooflines(stats, T, V, nnzb, prec, bf16=True):
                            "CUDA events around the plain F passes of one preconditioner application per step "
                            "(median over the steps); launches per step = (F steps - 1) x Arnoldi steps",
                  "algorithmic_bytes_per_launch": int(f_bytes)}
+        if cycle:
+            fpass["note"] = reuse
     # Krylov SpMV (inner FP32 in mixed precision, FP64 otherwise)
     spmv_ms = sum(s["ms_spmv"] for s in stats) / max(1, sum(s["n_spmv"] for s in stats))
     sv = 4 if dd else 8
@@ -239,7 +245,7 @@ def kernel_rooflines(stats, T, V, nnzb, prec, bf16=True):
             "traffic": int(SPMV32_DRAM_BYTES_PER_BLOCK * nnzb) if sv == 4 and not cycle else None, "peak_source": src + " (burst copy)",
             "ms_per_launch": round(spmv_ms, 5), "launches_per_step": round(its, 1),
             "ms_per_step": round(spmv_ms * its, 4),
-            "timing": clock + "; products per step = Arnoldi steps" if cycle else
+            "timing": clock_product + "; products per step = Arnoldi steps" if cycle else
                       "CUDA events around one Arnoldi SpMV launch in five (at most 4 per step); launches "
                       "per step = Arnoldi steps",
             "algorithmic_bytes_per_launch": int(spmv_bytes)}

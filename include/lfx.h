@@ -325,8 +325,9 @@ typedef struct lfx_step_stats {
   int32_t n_assembly_launches;  /* launches of the assembly kernel in this step: element colours,
                                    chunk colours, or 1 for the persistent launch                */
   float ms_spmv;                /* device time of Arnoldi block products of the (inner) Krylov solve
-                                   in this step: all of them where the persistent cycle runs (its own
-                                   clock), else a sample, one in five, at most four (CUDA events)  */
+                                   in this step: all of them where the persistent cycle runs (each the
+                                   slowest CTA's time, without the grid-wide wait that follows), else a
+                                   sample, one in five, at most four (CUDA events)                */
   int32_t n_spmv;               /* their number (FP64 matrix on the FP64 path, FP32 in mixed)   */
   int32_t newton_iterations;    /* Newton updates taken (fully implicit formulation), else 0    */
   float ms_newton_assembly;     /* device time of the Newton loop's assemblies: the residual

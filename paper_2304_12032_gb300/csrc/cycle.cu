@@ -775,6 +775,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ T hs[kMaxRestart + 1];
   __shared__ SumT red[(kMaxRestart + 1) * kDots];
+  __shared__ unsigned long long t0, ns_f;   // thread 0's clock and sum (in registers they would be every thread's)
   __shared__ int verdict, resident, solved, over;   // over: this CTA's segment has converged (thread 0's)
   if (finished(A.ks)) return;
   const unsigned rows_ctas = gridDim.x - 1, cta = blockIdx.x;
@@ -856,6 +857,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
   __syncthreads();
   if (tid == 0) {   // rows whose velocity records fit
     over = 0;
+    ns_f = 0;
     const int64_t most = A.f_bytes / (12 * sizeof(S));
     int lo = 0, hi = o.n;
     while (lo < hi) {
@@ -917,8 +919,7 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
   T *const dbuf[2] = {A.D0, A.D1};
   const int decide_at = min(3, A.f_steps - 1);
   T s = T(1);                        // 1 / norm of the Krylov vector held in w
-  unsigned long long t0 = 0, ns_f = 0, ns_p = 0;
-  int j = 0, n_p = 0;
+  int j = 0;
   for (;; ++j) {
     // ---- z_u* ~= F^-1 v_u: Chebyshev steps; the first one reads diag(F)^-1 w
     for (int k = 1; k < A.f_steps; ++k) {
@@ -1090,14 +1091,11 @@ __global__ void __launch_bounds__(Shape<T, LPR>::threads, 1) cycle_kernel(const 
     }
     LFX_CYCLE_SYNC();
     // ---- w = A z, then its products with the basis (own rows only: no barrier between)
-    if (cta == 0 && tid == 0) t0 = now_ns();
+    if (tid == 0) t0 = now_ns();
     load4(zj);
     R::product(o, A.A, A.lcol);
     __syncthreads();
-    if (cta == 0 && tid == 0) {
-      ns_p += now_ns() - t0;
-      ++n_p;
-    }
+    if (tid == 0) atomicMax(&A.sync->product_ns[j], (unsigned)(now_ns() - t0));
     const int nv = j + 1;
     {
       const int shares = max(1, min(kDots, NW / nv));
@@ -1196,6 +1194,14 @@ ended:
   }
   __syncthreads();
   if (!solved) return;
+  if (cta == 0 && tid == 0) {
+    unsigned long long ns_p = 0;
+    for (int i = 0; i < j; ++i) ns_p += A.sync->product_ns[i];
+    A.sync->t_f += ns_f;
+    A.sync->n_f += (A.f_steps - 2) * j + max(decide_at - 2, 0);   // (with those of the step the verdict interrupted)
+    A.sync->t_spmv += ns_p;
+    A.sync->n_spmv += j;
+  }
   const KState *own = A.n_seg > 1 ? A.kseg + A.cta_seg[cta] : A.ks;
   if (A.n_seg > 1) j = own->j;   // (steps until this segment had converged)
   for (int i = tid; i < j; i += NT) hs[i] = (T)own->y[i];
@@ -1212,12 +1218,6 @@ ended:
       a.w += y * z.w;
     }
     st4(A.x, r0 + e, a);
-  }
-  if (cta == 0 && tid == 0) {
-    A.sync->t_f += ns_f;
-    A.sync->n_f += (A.f_steps - 2) * n_p;
-    A.sync->t_spmv += ns_p;
-    A.sync->n_spmv += n_p;
   }
 #undef LFX_CYCLE_SYNC
 }

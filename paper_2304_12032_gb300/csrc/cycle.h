@@ -24,8 +24,11 @@ struct CycleSync {
   unsigned arrived;       // arrivals at the grid barrier, all steps
   unsigned progress;      // 2 (steps decided) + (1 if the cycle has ended)
   unsigned solved;        // 1 once y = R^-1 g is in place
+  unsigned product_ns[kMaxRestart];   // the slowest CTA's time in the product of each step (statistics)
   int error;              // a bounded wait gave up
-  unsigned long long t_f, t_spmv;   // nanoseconds of CTA 0 in plain F passes and products (statistics)
+  // statistics of the cycles since the last check: nanoseconds of plain F passes (from barrier to barrier) and
+  // of products (the slowest CTA's, summed), and their numbers
+  unsigned long long t_f, t_spmv;
   int n_f, n_spmv;
 };
 

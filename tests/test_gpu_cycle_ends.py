@@ -73,3 +73,16 @@ def test_hard_member_beside_easy_ones(precision):
         assert rel(u[sl], ui) < 1e-7 and rel(p[sl], pi) < 1e-7
     assert min(steps) < max(steps)
     assert stats["iterations"] <= 1.25 * max(steps) + 4
+
+
+@pytest.mark.parametrize("f_steps,more", [(2, 0), (3, 0), (4, 1), (6, 1)])
+def test_cycle_statistics_count_what_was_timed(f_steps, more):
+    """One product per Arnoldi step; the plain velocity passes of every step (all but the first), and those of the
+    last, unfinished step before the verdict that ends a cycle (two cycles here)."""
+    case = C.beltrami_case(9, seed=9)
+    _, _, st = C.gpu_state(case, gmres_rtol=1e-30, gmres_restart=6, gmres_max_iters=12, f_steps=f_steps)
+    stats = st.step(allow_not_converged=True)
+    assert stats["iterations"] == 12 == stats["n_spmv"]
+    assert stats["n_fpass"] == (f_steps - 2) * 12 + 2 * more
+    assert 0.0 < stats["ms_spmv"] < stats["ms_solve"]
+    assert stats["n_fpass"] * stats["ms_fpass_median"] < stats["ms_solve"]
