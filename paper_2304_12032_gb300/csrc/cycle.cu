@@ -487,7 +487,7 @@ struct Rows<double, LPR> {
     }
   }
   static __device__ __forceinline__ void product(const Own<double> &o, const double *A, const uint16_t *lcol) {
-    constexpr int W = SUB == 1 ? 2 : 2;
+    constexpr int W = 2;   // blocks in flight per lane
     const int tid = pass_tid(), lane = tid % LPR, comp = lane & 3, sub = lane >> 2;
 #pragma unroll 1
     for (int base = 0; base < o.n; base += NT / LPR) {

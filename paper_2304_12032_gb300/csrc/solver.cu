@@ -2460,10 +2460,10 @@ lfx_status ASimple<S, T>::setup_view(cudaStream_t st, const View &A) {
       pdl_launch(bound64_kernel<View, 1>, g3, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>());
       pdl_launch(bound64_kernel<View, 2>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>());
     } else {
-    pdl_launch(bound_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>(), 0);
-    pdl_launch(reduce_kernel, 1, kThreads, 0, st, part.as<double>(), rg, lam_f, 2);
-    pdl_launch(bound_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>(), 1);
-    pdl_launch(bound_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>(), 2);
+      pdl_launch(bound_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>(), 0);
+      pdl_launch(reduce_kernel, 1, kThreads, 0, st, part.as<double>(), rg, lam_f, 2);
+      pdl_launch(bound_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>(), 1);
+      pdl_launch(bound_kernel<View, T>, rg, kThreads, 0, st, A, dinvF.as<T>(), dinvS.as<T>(), W.as<T>(), part.as<double>(), 2);
     }
     pdl_launch(reduce_kernel, 1, kThreads, 0, st, part.as<double>(), rg, lam_s, 2);
     note_launches(5);
