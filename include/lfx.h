@@ -262,16 +262,19 @@ typedef struct lfx_options {
    * colour, each CTA scattering its elements' blocks), LFX_ASM_CHUNKS (compact 32-element chunks,
    * their blocks reduced in shared memory and written once per chunk, one launch per chunk colour),
    * LFX_ASM_PERSISTENT (the chunks in one cooperative launch, colours separated by bounded grid-wide
-   * waits, or, on meshes of up to about 190k tetrahedra, all chunks at once into a scratch and one wait
-   * before each block is summed over its chunks; LFX_ERR_TIMEOUT from lfx_step if a wait gives up), or LFX_ASM_AUTO (default): the first
+   * waits, or, on meshes of up to about 190k tetrahedra, all chunks at once into a scratch (about 0.8 KB
+   * per tetrahedron and state, where it can be had) and one wait before each block is summed over its
+   * chunks; LFX_ERR_TIMEOUT from lfx_step if a wait gives up), or LFX_ASM_AUTO (default): the first
    * assembly on the problem times each of the three on the device (two assemblies each) and the
    * problem keeps the fastest for all its states (lfx_problem_assembly_tuning reports it).  The
    * Newton system of the fully implicit formulation is timed and chosen apart from it, at its own
    * first assembly, since its kernels fit the SMs differently. */
   int32_t assembly;
   double newton_rtol;           /* default 1e-10                                                 */
-  /* velocity smoothing passes of the BF16 smoother (smoother_bf16 = 1): 1 (default) the staged
-   * pass, whose persistent CTAs copy whole row tiles of F sub-blocks into shared memory with bulk
+  /* velocity smoothing passes of the BF16 smoother (smoother_bf16 = 1) in solves that run step by
+   * step (a second Gram-Schmidt pass, resistance outlets, other Schur smoothing than one AMG V-cycle,
+   * sizes past the persistent Krylov cycle's shared memory; the cycle has passes of its own): 1
+   * (default) the staged pass, whose persistent CTAs copy whole row tiles of F sub-blocks into shared memory with bulk
    * asynchronous copies while the previous tile is processed (LFX_ERR_TIMEOUT from lfx_step if a
    * bounded wait for a tile gives up); 0 the plain pass, each lane loading its blocks itself.  Both
    * compute the same sums in the same order. */
@@ -532,7 +535,8 @@ lfx_status lfx_problem_state_bytes(const lfx_problem *problem, int64_t *bytes);
  * Serving (not in the paper): continuous batching of independent simulations on one GPU.
  * Requests wait FIFO until the device-memory budget admits them; admitted simulations keep
  * their state resident, each on its own stream, and n_workers host threads step them
- * round-robin one step at a time, so kernels of different simulations overlap.  When one
+ * round-robin one step at a time, so kernels of different simulations overlap (persistent Krylov
+ * cycles, which take every SM, run one after another).  When one
  * finishes, its result is copied to host memory, its device memory released and waiting
  * requests are admitted.  Results are independent of the mix (no shared reductions).
  * ------------------------------------------------------------------------------------------ */
@@ -560,7 +564,8 @@ void lfx_server_destroy(lfx_server *server);
 
 /* One step of each of n independent simulations (distinct states, each on its own stream set
  * with lfx_set_stream; states on the same stream run one after another): the steps run
- * concurrently, one host thread per state, so their kernels overlap on the device; stats [n]
+ * concurrently, one host thread per state, so their kernels overlap on the device (persistent Krylov
+ * cycles, which take every SM, run one after another); stats [n]
  * (nullable) receive each step's statistics.  Returns LFX_OK, or the first failure in state order
  * (a hard error before LFX_ERR_NOT_CONVERGED), with the state's index in lfx_last_error().
  * Every state has advanced unless its own step failed.  Many small meshes are batched more tightly

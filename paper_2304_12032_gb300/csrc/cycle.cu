@@ -17,8 +17,11 @@
 // 500k mixed 16.1 and 10.9, 600k FP64 48.4 and 33.2, 1.02M mixed 24.1 and 17.9.  A pass costs 1.4 us for the
 // barrier (waiting for the halo's CTAs only: 2 us, their flags arrive one by one), 1.1 to 1.7 us of latency
 // (neighbour copy, records, sums) at 32 rows per CTA, and then grows with the rows: at 1M tetrahedra 14 us per
-// velocity pass and 7 us per gradient or divergence pass, bound by L1 line lookups of the record loads.
-// FP64 passes run at the FP64 pipe's rate (a velocity pass at 108k nodes: 45 us, 37 us of it FP64 issue).
+// velocity pass and 7 us per gradient or divergence pass.  No unit is full there (over a launch at 818k the L1 data
+// pipe is 46 % busy, issue 28 %, DRAM 21 %): barrier, halo copy and the first record loads follow one another.
+// FP64 passes run at the FP64 pipe's rate (a velocity pass at 108k nodes: 45 us, 37 us of it FP64 issue); with the
+// barriers the pipe is 50 % busy over a launch at 102k tetrahedra.  A system within amg_coarse_size has 11 passes
+// per step, the dense inverse among them (729 nodes, FP64: 3.9 us each).
 //
 // A batch of independent meshes runs the same way, each piece with CTAs, basis, sums and stopping test of its
 // own (16 meshes of 10k to 40k tetrahedra in one launch: 13.3 -> 8.0 ms a step).

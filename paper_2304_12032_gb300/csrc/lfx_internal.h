@@ -210,9 +210,11 @@ struct PhysParams {
 };
 
 constexpr int kChunkElems = 32;     // elements per chunk (one CTA pass of the assembly kernels)
-// Meshes of up to this many chunks are assembled by gathering (when the persistent launch is chosen):
-// below it the chunk colours hold fewer chunks than the GPU runs at once, so that colour by colour most
-// of it idles.  The scratch is about 26 KB per chunk (FP64 or double-float), 160 MB at the limit.
+// Meshes of up to this many chunks are assembled by gathering (when the persistent launch is chosen).  The
+// limit is the memory of the scratch: about 26 KB per chunk (FP64 or double-float), 160 MB per state at the
+// limit, where gathering still pays (assembly kernel, coloured and gathered, 152k tetrahedra: mixed 0.58 and
+// 0.42 ms, FP64 1.28 and 0.85; 194k: 0.59 and 0.52, 1.41 and 1.05).  What it saves is the waiting of a coloured launch whose
+// colours hold fewer chunks than the GPU runs at once, so it pays less the more chunks there are.
 constexpr int kGatherChunks = 6144;
 constexpr int kChunkMaxPasses = 8;  // passes of 4 kChunkElems slots a chunk may take (the kernels stage
                                     // a chunk's slot codes for this many in shared memory)
